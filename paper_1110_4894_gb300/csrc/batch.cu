@@ -84,18 +84,13 @@ __device__ __forceinline__ bool cone_active(const BatchCone &C, int step)
     return *(volatile unsigned long long *)&C.cnt[(step - 1) & 1] != 0ull;
 }
 
-__global__ void k_batch_schedule(BatchArgs B)
+// step table of cone blockIdx.y
+__global__ void __launch_bounds__(kSchedThreads) k_batch_schedule(BatchArgs B)
 {
     BatchCone &C = B.cones[blockIdx.y];
-    __shared__ double s_chi;
-    if (threadIdx.x == 0) {
-        s_chi = comoving_distance(C.tp.cosmo, C.z_s);
-        if (blockIdx.x == 0) C.chi_s = s_chi;
-    }
-    __syncthreads();
-    const int n = C.tp.n_steps;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
-        C.dlam[k] = schedule_step(C.tp.cosmo, C.kind, n, k, s_chi, C.chi_l, C.s_asinh);
+    const double chi_s = comoving_distance(C.tp.cosmo, C.z_s);
+    if (blockIdx.x == 0 && threadIdx.x == 0) C.chi_s = chi_s;
+    schedule_steps(C.tp.cosmo, C.kind, C.tp.n_steps, chi_s, C.chi_l, C.s_asinh, C.dlam);
 }
 
 __global__ void k_batch_init(BatchArgs B)
@@ -308,9 +303,8 @@ cudaError_t batch_launch(const BatchArgs &B, int NT, int MODE, int grid, int max
 {
     cudaError_t e;
     {
-        int bx = (max_sched_steps + 127) / 128;
-        if (bx > 64) bx = 64;
-        k_batch_schedule<<<dim3((unsigned)std::max(bx, 1), (unsigned)B.n_cones), 128, 0, st>>>(B);
+        const int bx = std::max(1, std::min(max_sched_steps, 64));
+        k_batch_schedule<<<dim3((unsigned)bx, (unsigned)B.n_cones), kSchedThreads, 0, st>>>(B);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     k_batch_init<<<(unsigned)((B.T + 255) / 256), 256, 0, st>>>(B);

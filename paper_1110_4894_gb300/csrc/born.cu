@@ -18,10 +18,11 @@ namespace rt3d {
 __global__ void k_born_nodes(Cosmo c, double z_s, int kind, int n, double chi_l, double s, double *__restrict__ x,
                              double *__restrict__ w)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > n) return;
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) / kGroup;  // one lane group per node
     const double chi_s = comoving_distance(c, z_s);
-    const double xk = sched_node(kind, n, k, chi_s, chi_l, s);
+    const double xk = k <= n ? sched_node(kind, n, k, chi_s, chi_l, s) : 0.0;
+    const double zk = redshift_at(c, xk);
+    if (k > n || threadIdx.x % kGroup != 0) return;
     double du, jac;
     if (kind == RT3D_SCHED_UNIFORM) {
         du = chi_s / n;
@@ -32,7 +33,7 @@ __global__ void k_born_nodes(Cosmo c, double z_s, int kind, int n, double chi_l,
     }
     const double W = xk * (chi_s - xk) / chi_s;
     x[k] = xk;
-    w[k] = ((k == 0 || k == n) ? 0.5 : 1.0) * du * jac * W * (1.0 + redshift_at(c, xk));
+    w[k] = ((k == 0 || k == n) ? 0.5 : 1.0) * du * jac * W * (1.0 + zk);
 }
 
 // points of nodes [k0, k0 + K) for every bundle, node-major (neighbouring
@@ -227,7 +228,7 @@ cudaError_t born_run(const Cosmo &c, const DevField &f, int64_t n_particles, dou
     int *rep = (int *)(pts + 3 * m);
     float2 *part = (float2 *)(((uintptr_t)(rep + m) + 255) & ~(uintptr_t)255);
     cudaError_t e;
-    k_born_nodes<<<(n + 1 + 127) / 128, 128, 0, st>>>(c, z_s, kind, n, chi_l, s, x, w);
+    k_born_nodes<<<((n + 1) * kGroup + 127) / 128, 128, 0, st>>>(c, z_s, kind, n, chi_l, s, x, w);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(d_out, 0, sizeof(double) * 3 * n_b, st)) != cudaSuccess) return e;
     const int64_t tiles = std::max<int64_t>(1, (n_particles + kTile - 1) / kTile);

@@ -1,6 +1,8 @@
 // kernels.cu -- FP64 kernels of the trace: step schedule (cosmology
 // precompute), bundle initialiser, RK4 integrator stage, bundle reducer,
 // muPDF histogram and particle staging.
+#include <algorithm>
+
 #include "trace_device.cuh"
 
 namespace rt3d {
@@ -8,9 +10,6 @@ namespace rt3d {
 // ---------------------------------------------------------------------------
 // background cosmology on the device (Sec. 3.5, Eq. raytracedistance)
 // ---------------------------------------------------------------------------
-// One block computes chi_s; every thread then fills dlam[k] = int a^2 dchi over
-// [x_k, x_{k+1}] (the affine step of the unperturbed ray with dx3/dl = 1 at the
-// observer), by composite Boole's rule with 4 panels.
 // a(t) and h da/dt at t = j h (the closed forms of Eq. scalefac2)
 __global__ void k_atab(Cosmo c, int n, double h, double *__restrict__ tab)
 {
@@ -27,26 +26,20 @@ cudaError_t launch_atab(const Cosmo &c, int n, double h, double *d_tab, cudaStre
     return cudaGetLastError();
 }
 
-__global__ void k_schedule(Cosmo c, double z_s, int kind, int n, double chi_l, double s, double *dlam,
-                           double *misc)
+// chi_s to misc[0] and the affine steps
+__global__ void __launch_bounds__(kSchedThreads) k_schedule(Cosmo c, double z_s, int kind, int n, double chi_l,
+                                                            double s, double *dlam, double *misc)
 {
-    __shared__ double s_chi;
-    if (threadIdx.x == 0) {
-        s_chi = comoving_distance(c, z_s);
-        if (blockIdx.x == 0) misc[0] = s_chi;
-    }
-    __syncthreads();
-    const double chi_s = s_chi;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
-        dlam[k] = schedule_step(c, kind, n, k, chi_s, chi_l, s);
+    const double chi_s = comoving_distance(c, z_s);
+    if (blockIdx.x == 0 && threadIdx.x == 0) misc[0] = chi_s;
+    schedule_steps(c, kind, n, chi_s, chi_l, s, dlam);
 }
 
 cudaError_t launch_schedule(const Cosmo &c, double z_s, int kind, int n, double chi_l, double s, double *d_dlam,
                             double *d_misc, cudaStream_t st)
 {
-    int blocks = (n + 127) / 128;
-    if (blocks > 1024) blocks = 1024;
-    k_schedule<<<blocks, 128, 0, st>>>(c, z_s, kind, n, chi_l, s, d_dlam, d_misc);
+    k_schedule<<<std::min(n, 16 * device_sm_count()), kSchedThreads, 0, st>>>(c, z_s, kind, n, chi_l, s, d_dlam,
+                                                                              d_misc);
     return cudaGetLastError();
 }
 

@@ -99,16 +99,13 @@ __device__ void plane_q_range(MPPlane &p, int replicated, int slices, double chi
 __global__ void k_mp_table(Cosmo c, DevField f, double z_s, int slices, double a_iso, double b_iso, int n_pl,
                            MPPlane *pl, double *misc)
 {
-    __shared__ double s_chi;
-    if (threadIdx.x == 0) {
-        s_chi = comoving_distance(c, z_s);
-        misc[0] = s_chi;
-    }
-    __syncthreads();
-    const double chi_s = s_chi;
+    const double chi_s = comoving_distance(c, z_s);
+    if (threadIdx.x == 0) misc[0] = chi_s;
     const int replicated = f.replicated;
     const double L = f.L;
-    for (int q = threadIdx.x; q < n_pl; q += blockDim.x) {
+    // one lane group per plane (redshift_at is a whole-warp call)
+    for (int q0 = 0; q0 < n_pl; q0 += blockDim.x / kGroup) {
+        const int q = q0 + threadIdx.x / kGroup;
         const int j = q / slices, s = q % slices;
         double a, b;
         if (replicated) {
@@ -127,7 +124,8 @@ __global__ void k_mp_table(Cosmo c, DevField f, double z_s, int slices, double a
         p.hi = hi;
         p.thick = hi - lo;
         p.chi = 0.5 * (lo + hi);
-        p.zp1 = 1.0 + redshift_at(c, p.chi);
+        p.zp1 = 1.0 + redshift_at(c, q < n_pl ? p.chi : 0.0);
+        if (q >= n_pl || threadIdx.x % kGroup != 0) continue;
         p.a = a;
         p.b = b;
         p.d = d;
