@@ -165,7 +165,7 @@ struct rt3d_ctx {
     int tev_used = 0;
     double *atab = nullptr;  // a(t) table of the cosmology (device)
     size_t atab_n = 0;
-    unsigned long long *d_hist_u64 = nullptr;  // bins*2 + 5
+    unsigned long long *d_hist_u64 = nullptr;  // bins*2 + kHistScal
     double *d_hist_f64 = nullptr;              // 8
     int hist_cap = 0;
     double *d_io = nullptr;                    // staging for potential / histogram inputs
@@ -1666,7 +1666,7 @@ static int ensure_hist(rt3d_ctx *ctx, int bins)
         ctx->d_hist_u64 = nullptr;
         ctx->d_hist_f64 = nullptr;
         ctx->hist_cap = 0;
-        CK(cudaMalloc((void **)&ctx->d_hist_u64, (2 * (size_t)bins + 8) * sizeof(unsigned long long)));
+        CK(cudaMalloc((void **)&ctx->d_hist_u64, (2 * (size_t)bins + kHistScal) * sizeof(unsigned long long)));
         CK(cudaMalloc((void **)&ctx->d_hist_f64, 8 * sizeof(double)));
         ctx->hist_cap = bins;
     }

@@ -326,6 +326,9 @@ inline double partial_mass_factor(const DevField &f, const ForceShape &sh)
 }
 cudaError_t launch_reduce(const TraceParams &tp, const double *d_theta, RayState rs, const double *d_misc,
                           double *d_bout, double *d_rout, cudaStream_t st);
+// words of d_scal: five counters, a ticket, three doubles per block
+constexpr int kHistBlocks = 1024;
+constexpr int kHistScal = 6 + 3 * kHistBlocks;
 cudaError_t launch_histogram(int64_t n, const double *d_mu, int mu_stride, const int *d_flags,
                              const double *d_flagsd, int bins, double mu_min, double mu_max,
                              unsigned long long *d_counts, unsigned long long *d_wfix,
