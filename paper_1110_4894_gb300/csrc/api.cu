@@ -100,9 +100,13 @@ __global__ void k_stage_particles(int64_t n, const double *__restrict__ pos, con
     (void)soft0;
 }
 
-int force_max_splits(const ForceShape &, int64_t n_particles)
+// particles that a split's range is a multiple of: a tile of the FP32 sums; the
+// unroll of the FP64 sum, whose plain sums may be cut anywhere
+static int split_unit(const ForceShape &sh) { return sh.variant == 2 ? kUnit64 : kTile; }
+
+int force_max_splits(const ForceShape &sh, int64_t n_particles)
 {
-    const int64_t t = (n_particles + kTile - 1) / kTile;
+    const int64_t t = (n_particles + split_unit(sh) - 1) / split_unit(sh);
     return (int)std::max<int64_t>(1, std::min<int64_t>(t, 65535));
 }
 
@@ -648,9 +652,11 @@ static ForceShape choose_shape(rt3d_ctx *ctx, const DevField &f, int64_t n_point
         const int64_t tps = (tiles + S - 1) / S;
         S = (int)((tiles + tps - 1) / tps);
     } else {
-        // about five waves of resident blocks: many small blocks balance the
-        // SMs better than one exact wave
-        S = splits_for(nrb, (int64_t)ctx->n_sm * resident_blocks(f, sh), 5.0, tiles);
+        // FP32: about five waves of resident blocks, as many small blocks
+        // balance the SMs better than one exact wave of whole tiles.  FP64:
+        // one wave, which units of four particles fill evenly, and fewer
+        // partials to add up
+        S = splits_for(nrb, (int64_t)ctx->n_sm * resident_blocks(f, sh), fp64 ? 1.0 : 5.0, tiles);
     }
     sh.splits = std::max(1, S);
     // the expanded two-bundle kernel can add groups of 4 splits in a cluster
@@ -662,8 +668,8 @@ static ForceShape choose_shape(rt3d_ctx *ctx, const DevField &f, int64_t n_point
 
 static int64_t per_split_of(const ForceShape &sh, int64_t n_particles)
 {
-    const int64_t tiles = std::max<int64_t>(1, (n_particles + kTile - 1) / kTile);
-    return ((tiles + sh.splits - 1) / sh.splits) * kTile;
+    const int64_t unit = split_unit(sh), units = std::max<int64_t>(1, (n_particles + unit - 1) / unit);
+    return ((units + sh.splits - 1) / sh.splits) * unit;
 }
 
 static cudaError_t run_force(rt3d_ctx *ctx, const DevField &f, const double *px, const double *py, const double *pz,
@@ -2144,7 +2150,7 @@ extern "C" int rt3d_potential_device_noalloc(rt3d_ctx *ctx, void *stream, int fi
     // keep splits * 4 outputs * n points * 8 bytes inside the static array
     const int64_t cap = (int64_t)(RT3D_NOALLOC_SCRATCH_BYTES / ((size_t)32 * (size_t)n));
     if (sh.splits > cap) {
-        const int64_t tiles = std::max<int64_t>(1, (fs.n + kTile - 1) / kTile);
+        const int64_t tiles = force_max_splits(sh, fs.n);
         const int64_t tps = (tiles + cap - 1) / cap;
         sh.splits = (int)std::max<int64_t>(1, (tiles + tps - 1) / tps);
     }

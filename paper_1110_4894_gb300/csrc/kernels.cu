@@ -70,8 +70,8 @@ cudaError_t launch_init(const TraceParams &tp, const DevField &f, const double *
 // termination on x3 with linear interpolation: Sec. 3.4)
 // ---------------------------------------------------------------------------
 // A block of 256 threads serves 64 rays: first every thread reduces one
-// output of one ray's split partials (mixed precision: four threads per ray,
-// which keeps four times more loads in flight), then one thread per ray runs
+// output of one ray's split partials (four threads per ray, which keeps four
+// times more loads in flight), then one thread per ray runs
 // the FP64 stage update with whole warps active.
 constexpr int kStageRays = 64;
 // from this many rays on (four blocks of 256 per SM), one ray per thread
@@ -121,16 +121,18 @@ __global__ void __launch_bounds__(256) k_stage(TraceParams tp, DevField f, RaySt
     __shared__ unsigned s_active;
     if (threadIdx.x == 0) s_active = 0;
     const int64_t r0 = (int64_t)blockIdx.x * kStageRays;
-    if (!fp64) {
+    {
         const int local = threadIdx.x >> 2, o = threadIdx.x & 3;
         const int64_t i = r0 + local;
-        if (i < rs.n_rays) s_acc[local][o] = reduce_partials_mixed((const float2 *)partials, S, rs.n_rays, i, o);
+        if (i < rs.n_rays)
+            s_acc[local][o] = fp64 ? reduce_partials_fp64((const double *)partials, S, rs.n_rays, i, o)
+                                   : reduce_partials_mixed((const float2 *)partials, S, rs.n_rays, i, o);
     }
     __syncthreads();
     if (threadIdx.x < kStageRays) {
         const int64_t i = r0 + threadIdx.x;
         if (i < rs.n_rays && stage_ray(tp, f, rs, S, fp64 != 0, mfac, partials, dlam, misc[0], step, stage, cnt, i,
-                                       fp64 ? nullptr : s_acc[threadIdx.x], prism))
+                                       s_acc[threadIdx.x], prism))
             atomicAdd(&s_active, 1u);
     }
     __syncthreads();

@@ -264,6 +264,7 @@ __device__ __forceinline__ double reduce_partials_mixed(const float2 *__restrict
                                                         int o)
 {
     float hi = 0.0f, lo = 0.0f;
+#pragma unroll 8  // loads in flight ahead of the serial sum
     for (int s = 0; s < S; ++s) {
         const float2 v = pm[((int64_t)s * 4 + o) * n + i];
         const float t = hi + v.x;
@@ -273,6 +274,16 @@ __device__ __forceinline__ double reduce_partials_mixed(const float2 *__restrict
         lo += err + v.y;
     }
     return (double)hi + (double)lo;
+}
+
+// the same for FP64 partials: a plain sum in split order
+__device__ __forceinline__ double reduce_partials_fp64(const double *__restrict__ pd, int S, int64_t n, int64_t i,
+                                                       int o)
+{
+    double acc = 0.0;
+#pragma unroll 8
+    for (int s = 0; s < S; ++s) acc += pd[((int64_t)s * 4 + o) * n + i];
+    return acc;
 }
 
 // Reduce the pair-sum partials of one ray and add the mean subtraction:
