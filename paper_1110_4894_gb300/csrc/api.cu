@@ -959,6 +959,12 @@ static int trace_advance(rt3d_ctx *ctx, int n, cudaStream_t st)
     const int nr = T.rs.nr;
     Scratch &s = ctx->scr;
     const int stop = std::min(T.total, T.next + n);
+    if (fs.is_grid && !T.timed && T.next < stop) {  // all the stages in one launch (timed traces: kernel by kernel)
+        CK(launch_grid_trace(T.tp, fs.gd, T.rs, T.fp64, T.next, stop, s.dlam, s.misc, s.counters, st));
+        T.next = stop;
+        T.launches += 1;
+        T.flaunch += 1;
+    }
     for (; T.next < stop; ++T.next) {
         const int g = T.next, step = g / 4, stage = g % 4;
         // extra steps past the table run only while some ray is not across

@@ -47,32 +47,33 @@ __device__ __forceinline__ void spline_weights_f(float u, float (&c)[W])
     }
 }
 
-// phi and grad phi (F[0..3]) at point i from the FP32 node table: App. B's
+// The cube of box grids that holds x3 (the one of a bundle's central ray): its
+// corner replaces lo; returns its index among the node tables (0 for an
+// isolated grid).
+__device__ __forceinline__ int64_t grid_cube(const GridDev &g, double x3, double lo[3])
+{
+    if (g.cubes <= 0) return 0;
+    double q = floor(x3 / g.L);
+    const int j = q < 0.0 ? 0 : (q > (double)(g.n_rep - 1) ? g.n_rep - 1 : (int)q);
+    double cq = floor((x3 - (double)j * g.L) / g.W);
+    const int c = cq < 0.0 ? 0 : (cq > (double)(g.cubes - 1) ? g.cubes - 1 : (int)cq);
+    lo[0] = -0.5 * g.W;
+    lo[1] = -0.5 * g.W;
+    lo[2] = (double)j * g.L + (double)c * g.W;
+    return (int64_t)j * g.cubes + c;
+}
+
+// phi and grad phi (F[0..3]) at position r from the FP32 node table: App. B's
 // interpolation with FP32 weights and sums; the cube (box grids: the one
-// holding the x3 of the first point of i's group, the bundle's central ray),
-// node window and fractional offsets come from FP64 coordinates.  Zero
-// outside the node range widened by g.margin.
+// holding x3, the central ray's), node window and fractional offsets come from
+// FP64 coordinates.  Zero outside the node range widened by g.margin.
 template <int NI>
-__device__ __forceinline__ void grid_eval32_point(const GridDev &g, const double *__restrict__ px,
-                                                  const double *__restrict__ py, const double *__restrict__ pz,
-                                                  int64_t i, int group, float F[4])
+__device__ __forceinline__ void grid_eval32_at(const GridDev &g, const double r[3], double x3, float F[4])
 {
     constexpr int W = 2 * NI;
     const int n = g.n;
-    const double r[3] = {px[i], py[i], pz[i]};
     double lo[3] = {g.lo[0], g.lo[1], g.lo[2]};
-    const float *tab = g.tab32;
-    if (g.cubes > 0) {
-        const double x3 = pz[(i / group) * group];
-        double q = floor(x3 / g.L);
-        const int j = q < 0.0 ? 0 : (q > (double)(g.n_rep - 1) ? g.n_rep - 1 : (int)q);
-        double cq = floor((x3 - (double)j * g.L) / g.W);
-        const int c = cq < 0.0 ? 0 : (cq > (double)(g.cubes - 1) ? g.cubes - 1 : (int)cq);
-        lo[0] = -0.5 * g.W;
-        lo[1] = -0.5 * g.W;
-        lo[2] = (double)j * g.L + (double)c * g.W;
-        tab += ((int64_t)j * g.cubes + c) * kGridRec * (int64_t)n * n * n;
-    }
+    const float *tab = g.tab32 + grid_cube(g, x3, lo) * (kGridRec * (int64_t)n * n * n);
     double u[3];
     int s[3];
     bool inside = true;
@@ -115,6 +116,17 @@ __device__ __forceinline__ void grid_eval32_point(const GridDev &g, const double
 #pragma unroll
         for (int f = 0; f < 4; ++f) F[f] += c2[b] * acc[f];
     }
+}
+
+// the same at point i of the arrays; the cube is that of the first point of
+// i's group (a bundle's central ray)
+template <int NI>
+__device__ __forceinline__ void grid_eval32_point(const GridDev &g, const double *__restrict__ px,
+                                                  const double *__restrict__ py, const double *__restrict__ pz,
+                                                  int64_t i, int group, float F[4])
+{
+    const double r[3] = {px[i], py[i], pz[i]};
+    grid_eval32_at<NI>(g, r, g.cubes > 0 ? pz[(i / group) * group] : 0.0, F);
 }
 
 // grid_eval32_point for the grid's n_int (1..4)

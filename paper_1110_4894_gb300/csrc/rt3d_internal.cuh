@@ -383,6 +383,10 @@ cudaError_t launch_grid_eval(const GridDev &g, const double *px, const double *p
                              int mode, void *out, const unsigned long long *gate, cudaStream_t st,
                              int group = 1);
 
+// RK4 stages [g0, g1) of a trace on a grid in one launch
+cudaError_t launch_grid_trace(const TraceParams &tp, const GridDev &g, const RayState &rs, bool fp64, int g0, int g1,
+                              const double *dlam, const double *misc, unsigned long long *cnt, cudaStream_t st);
+
 // Born approximation (born.cu): scratch size and the run over node chunks of
 // K nodes with the Hessian pair sum split `splits` ways; d_out = n_b x 3
 size_t born_scratch_bytes(int64_t n_b, int n_steps, int K, int splits);

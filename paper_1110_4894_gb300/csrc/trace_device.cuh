@@ -347,6 +347,24 @@ __device__ __forceinline__ void geodesic_rhs(const double y[8], const double F[4
     k[7] = -gz * tt - drag * vz - ia * (gz * v2 - 2.0 * vz * gv);
 }
 
+// d y / d lambda at stage state ys with the field F; at the observer (first)
+// dt/dl of ys and of the step's state y is set from the null condition.
+__device__ __forceinline__ void ray_slope(const TraceParams &tp, double ys[8], const double F[4], bool first,
+                                          double y[8], double k[8])
+{
+    const double a = cosmo_a(tp.cosmo, ys[0]);
+    const double ia = 1.0 / a;
+    const double ad = cosmo_adot_ia(tp.cosmo, a, ia);
+    if (first) {
+        // null condition of Eq. expandingmetric with psi = phi / a
+        const double vn = sqrt(ys[5] * ys[5] + ys[6] * ys[6] + ys[7] * ys[7]);
+        const double T = a * vn * sqrt((1.0 - 2.0 * F[0] / a) / (1.0 + 2.0 * F[0] / a));
+        ys[4] = T;
+        y[4] = T;
+    }
+    geodesic_rhs(ys, F, a, ia, ad, tp.christoffel, k);
+}
+
 // One ray's RK4 stage: gather phi and grad phi, set dt/dl from the null
 // condition at the observer, evaluate the geodesic right-hand side, update the
 // stage state or (stage 3) combine, terminate and interpolate.  rs is a view:
@@ -373,18 +391,8 @@ __device__ __forceinline__ bool stage_ray(const TraceParams &tp, const DevField 
     const double *rec = prism ? prism + kPrismRec * b : nullptr;
     if (pre) field_from_sums(f, pre, rep, ys + 1, mfac, F, rec);
     else gather_field(f, S, fp64, partials, rs.n_rays, i, rep, ys + 1, mfac, F, rec);
-    const double a = cosmo_a(tp.cosmo, ys[0]);
-    const double ia = 1.0 / a;
-    const double ad = cosmo_adot_ia(tp.cosmo, a, ia);
-    if (step == 0 && stage == 0) {
-        // null condition of Eq. expandingmetric with psi = phi / a
-        const double vn = sqrt(ys[5] * ys[5] + ys[6] * ys[6] + ys[7] * ys[7]);
-        const double T = a * vn * sqrt((1.0 - 2.0 * F[0] / a) / (1.0 + 2.0 * F[0] / a));
-        ys[4] = T;
-        y[4] = T;
-        rs.y[4 * st + i] = T;
-    }
-    geodesic_rhs(ys, F, a, ia, ad, tp.christoffel, k);
+    ray_slope(tp, ys, F, step == 0 && stage == 0, y, k);
+    if (step == 0 && stage == 0) rs.y[4 * st + i] = y[4];
     const double dl = dlam[step < tp.n_steps ? step : tp.n_steps - 1];
     const int done = rs.done[i];
     double nx[8];
