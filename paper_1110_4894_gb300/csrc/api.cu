@@ -22,6 +22,7 @@ cudaError_t dispatch_bundle(const ForceArgs &A, const ForceShape &sh, bool umass
 cudaError_t dispatch_bundle2(const ForceArgs &A, const ForceShape &sh, bool umass, cudaStream_t st);
 cudaError_t dispatch_bundle2x(const ForceArgs &A, const ForceShape &sh, bool umass, cudaStream_t st,
                               int *occ = nullptr);
+cudaError_t dispatch_lanes(const ForceArgs &A, const ForceShape &sh, bool umass, cudaStream_t st);
 struct BatchArgs;
 
 // rays covered by one block of the pair-sum kernel of shape sh
@@ -607,6 +608,21 @@ static void round_to_clusters(ForceShape &sh)
     if (sh.cl > 1) sh.splits = (sh.splits + sh.cl - 1) / sh.cl * sh.cl;
 }
 
+// Whether the one-ray-per-lane kernel is the faster one for n_b bundles and
+// `tiles` splits of one tile: cycles per particle of a scheduler's share of the
+// warps.  Measured per particle: one-ray lanes 20 a warp; two-bundle threads
+// 200 while a scheduler has one warp of them (the chain of one iteration), 129
+// per warp beyond (the FP32 pipe), for rings of 4; for rings of 8 twice that.
+static bool lanes_faster(const rt3d_ctx *ctx, const ForceShape &sh, int64_t n_b, int tiles)
+{
+    const int64_t sched = 4 * (int64_t)ctx->n_sm;
+    const int64_t per_block = sh.R == 5 ? 25 : 14;
+    const int64_t w1 = (4 * ((n_b + per_block - 1) / per_block) * tiles + sched - 1) / sched;
+    const int64_t w2 = ((n_b + 2 * sh.NT - 1) / (2 * sh.NT) * (sh.NT / 32) * tiles + sched - 1) / sched;
+    const int64_t k = sh.R == 5 ? 1 : 2;
+    return 20 * w1 < k * (w2 <= 1 ? 200 : 129 * w2);
+}
+
 // ---------------------------------------------------------------------------
 // launch shape
 // ---------------------------------------------------------------------------
@@ -663,6 +679,9 @@ static ForceShape choose_shape(rt3d_ctx *ctx, const DevField &f, int64_t n_point
     // (off unless asked for: measured slower on the NFW workload, see the tuner)
     sh.cl = (sh.variant == 5 && group == 5 && ctx->opt.cluster == 4) ? 4 : 1;
     round_to_clusters(sh);
+    // (a launch shape that was asked for is kept)
+    sh.lanes = sh.variant == 5 && sh.cl == 1 && sh.splits == tiles && ctx->opt.splits <= 0 &&
+               ctx->opt.threads_per_block <= 0 && lanes_faster(ctx, sh, n_points / group, tiles);
     return sh;
 }
 
@@ -693,7 +712,8 @@ static cudaError_t run_force(rt3d_ctx *ctx, const DevField &f, const double *px,
     if (sh.variant == 1) return dispatch_mixed(A, sh, st);
     if (sh.variant == 3) return dispatch_bundle(A, sh, sh.umass != 0, st);
     if (sh.variant == 4) return dispatch_bundle2(A, sh, sh.umass != 0, st);
-    if (sh.variant == 5) return dispatch_bundle2x(A, sh, sh.umass != 0, st);
+    if (sh.variant == 5)
+        return sh.lanes ? dispatch_lanes(A, sh, sh.umass != 0, st) : dispatch_bundle2x(A, sh, sh.umass != 0, st);
     return dispatch_packed(A, sh, sh.umass != 0, st);
 }
 
@@ -728,7 +748,8 @@ static int tuned_shape(rt3d_ctx *ctx, const FieldSlot &fs, const double *px, con
                        const int *rep, int group, int64_t n, bool fp64, cudaStream_t st, ForceShape &out)
 {
     ForceShape base = choose_shape(ctx, fs.df, n, fp64, group);
-    if (!ctx->opt.autotune || ctx->opt.rays_per_thread > 0 || ctx->opt.threads_per_block > 0 || ctx->opt.splits > 0) {
+    // (a launch that small has one shape: nothing to time)
+    if (base.lanes || !ctx->opt.autotune || ctx->opt.rays_per_thread > 0 || ctx->opt.threads_per_block > 0 || ctx->opt.splits > 0) {
         out = base;
         return RT3D_OK;
     }

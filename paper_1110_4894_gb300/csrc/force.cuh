@@ -1094,6 +1094,133 @@ __global__ void __launch_bounds__(NT, TPSM / NT) k_force_bundle2x(ForceArgs A)
                                                             split, (float2 *)A.out, s_a, s_b, s_e, s_hl);
 }
 
+// The expanded sums of bundle2x_block_sum with one ray per lane, for launches
+// too small to fill the GPU with two-bundle threads.  There, a tile of 256
+// particles is one chain of 256 x ~200 cycles per thread (all ten rays of its
+// two bundles), and the launch lasts as long as that chain, however few bundles
+// there are: 25 us for 4 bundles and 5000 particles.  A lane with one ray has
+// a tenth of the work per particle and runs at ~25 cycles: 8.5 us for the same
+// launch, 38.6 -> 18.5 ms for 200 steps.  The central ray's
+// separation is formed in every lane of its bundle; each lane's operations,
+// their order and the anchor (the first central ray of the lane's group of
+// `group` bundles, the bundles of a two-bundle block) are those of the
+// two-bundle kernel, so the results are the same bits.  One tile per block
+// (blockIdx.y); a block holds NT / NR whole bundles.
+template <int NT, int NRING, bool REPL, bool PEPS, bool UMASS>
+__global__ void __launch_bounds__(NT) k_force_bundle1(ForceArgs A, int group)
+{
+    if (A.gate && *A.gate == 0ull) return;
+    constexpr int NR = NRING + 1, BPB = NT / NR;
+    __shared__ float4 s_p[kTile];
+    __shared__ float s_e[PEPS ? kTile : 1];
+    __shared__ float4 s_c[BPB];
+    __shared__ int s_rmin, s_rmax;
+    const DevField &f = A.f;
+    const int tid = threadIdx.x, split = blockIdx.y;
+    const int per_group = (group + BPB - 1) / BPB;
+    const int64_t g0 = (int64_t)(blockIdx.x / per_group) * group;  // the group's first bundle
+    const int first = (int)(blockIdx.x % per_group) * BPB;         // the block's first bundle in the group
+    const int64_t n_b = A.n / NR;
+    const int g = tid % NR, lb = tid / NR;
+    const int64_t b = g0 + first + lb;
+    const bool valid = lb < BPB && first + lb < group && b < n_b;
+    if (tid == 0) {
+        s_rmin = INT_MAX;
+        s_rmax = INT_MIN;
+    }
+    __syncthreads();
+    const int myrep = valid ? checked_replica(A.rep ? A.rep[b] : 0, f.n_rep) : -1;
+    if (myrep >= 0) {
+        atomicMin(&s_rmin, myrep);
+        atomicMax(&s_rmax, myrep);
+    }
+    __syncthreads();
+    const int rmin = s_rmin, rmax = s_rmax;
+    const int64_t ic = b * NR, ia = g0 * NR;
+    float fx = 0.f, fy = 0.f, fz = 0.f, ee = 0.f;  // 2 e_k and |e_k|^2 (the central ray: zero)
+    if (valid && g > 0) {
+        const float vx = (float)(A.px[ic] - A.px[ic + g]), vy = (float)(A.py[ic] - A.py[ic + g]),
+                    vz = (float)(A.pz[ic] - A.pz[ic + g]);
+        fx = 2.f * vx;
+        fy = 2.f * vy;
+        fz = 2.f * vz;
+        ee = fmaf(vx, vx, fmaf(vy, vy, vz * vz));
+    }
+    float hx = 0.f, hy = 0.f, hz = 0.f, hs = 0.f, lx = 0.f, ly = 0.f, lz = 0.f, ls = 0.f, phi = 0.f;
+    const float dlt = (float)f.delta;
+    const int64_t p0 = (int64_t)split * kTile;
+    const int cnt = (int)min((int64_t)kTile, f.n - p0);
+    for (int j = rmin; j <= rmax; ++j) {
+        if (!__syncthreads_or(myrep == j)) continue;  // no point of this block is in replica j
+        double o[3];
+        frame_origin(f, j, o);
+        const long long ax = anchor_q(A.px[ia], o[0], f.inv_delta);
+        const long long ay = anchor_q(A.py[ia], o[1], f.inv_delta);
+        const long long az = anchor_q(A.pz[ia], o[2], f.inv_delta);
+        float nx = -1e30f, ny = -1e30f, nz = -1e30f;  // far sentinel
+        if (valid && myrep == j) {
+            nx = -(float)(((A.px[ic] - o[0]) * f.inv_delta - (double)ax) * f.delta);
+            ny = -(float)(((A.py[ic] - o[1]) * f.inv_delta - (double)ay) * f.delta);
+            nz = -(float)(((A.pz[ic] - o[2]) * f.inv_delta - (double)az) * f.delta);
+        }
+#pragma unroll 4
+        for (int q = tid; q < cnt; q += NT) {
+            const int4 pr = f.part[p0 + q];
+            long long qq[3] = {pr.x, pr.y, pr.z};
+            if (REPL) replica_q(f, j, pr.x, pr.y, pr.z, qq);
+            s_p[q] = make_float4((float)(qq[0] - ax) * dlt, (float)(qq[1] - ay) * dlt, (float)(qq[2] - az) * dlt,
+                                 __int_as_float(pr.w));
+            if (PEPS) s_e[q] = f.eps2[p0 + q];
+        }
+        __syncthreads();
+        float cx = 0.f, cy = 0.f, cz = 0.f, cs = 0.f;
+#pragma unroll 8
+        for (int jj = 0; jj < cnt; ++jj) {
+            const float4 a = s_p[jj];
+            const float e2 = PEPS ? s_e[jj] : f.eps2u;
+            const float dx = __fadd_rn(a.x, nx), dy = __fadd_rn(a.y, ny), dz = __fadd_rn(a.z, nz);
+            const float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, e2)));
+            const float w = rsqrt_mufu(__fadd_rn(r2, fmaf(fx, dx, fmaf(fy, dy, fmaf(fz, dz, ee)))));
+            const float u = __fmul_rn(w, w), mw = UMASS ? w : __fmul_rn(a.w, w), m3 = __fmul_rn(mw, u);
+            cs = __fadd_rn(cs, g == 0 ? mw : m3);  // the central ray's potential, a ring ray's S
+            cx = fmaf(dx, m3, cx);
+            cy = fmaf(dy, m3, cy);
+            cz = fmaf(dz, m3, cz);
+        }
+        __syncthreads();
+        if (g == 0) phi += cs;  // a bundle has one replica: a second pass adds zeros
+        two_sum_into(hx, lx, cx);
+        two_sum_into(hy, ly, cy);
+        two_sum_into(hz, lz, cz);
+        two_sum_into(hs, ls, cs);
+    }
+    if (valid && g == 0) s_c[lb] = make_float4(phi, hx + lx, hy + ly, hz + lz);
+    __syncthreads();
+    if (!valid) return;
+    if (g > 0) {  // G_k + e_k S_k as a (hi, lo) pair, and the potential to first order (ring_phi)
+        const float e[3] = {0.5f * fx, 0.5f * fy, 0.5f * fz};
+        float *hh[3] = {&hx, &hy, &hz}, *ll[3] = {&lx, &ly, &lz};
+#pragma unroll
+        for (int oo = 0; oo < 3; ++oo) {
+            const float hi = *hh[oo], p = e[oo] * hs;
+            const float pe = fmaf(e[oo], hs, -p);
+            const float sm = hi + p;
+            const float bv = sm - hi;
+            const float err = (hi - (sm - bv)) + (p - bv);
+            *ll[oo] = *ll[oo] + (err + fmaf(e[oo], ls, pe));
+            *hh[oo] = sm;
+        }
+        const float4 c = s_c[lb];
+        phi = ring_phi(c.x, e, c.y, c.z, c.w);
+    }
+    float2 *out = (float2 *)A.out;
+    const int64_t sn = (int64_t)split * 4, i = ic + g;
+    out[(sn + 0) * A.n + i] = make_float2(phi, 0.f);
+    out[(sn + 1) * A.n + i] = make_float2(hx, lx);
+    out[(sn + 2) * A.n + i] = make_float2(hy, ly);
+    out[(sn + 3) * A.n + i] = make_float2(hz, lz);
+}
+
 // ForceArgs for the bundle kernel: n = rays, group = rays per bundle; rep is
 // the per-bundle replica array.
 template <int NT, int NRING, bool REPL, bool PEPS, bool UMASS>

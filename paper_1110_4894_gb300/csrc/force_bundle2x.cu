@@ -65,6 +65,37 @@ static cudaError_t go_bundle2x8(const ForceArgs &A, dim3 grid, cudaStream_t st, 
     return go_fields<64, 8, UMASS, kRing8Threads, 1, kRing8Ahead>(A, grid, st, occ);
 }
 
+template <int NT, int NRING, bool UMASS>
+static cudaError_t go_lanes(const ForceArgs &A, int group, int splits, cudaStream_t st)
+{
+    const bool repl = A.f.replicated != 0, peps = A.f.eps2 != nullptr;
+    const int64_t n_b = A.n / (NRING + 1);
+    constexpr int BPB = NT / (NRING + 1);
+    // whole groups, then the blocks that the last group's bundles need
+    const int64_t full = n_b / group, rest = n_b % group;
+    const dim3 grid((unsigned)(full * ((group + BPB - 1) / BPB) + (rest + BPB - 1) / BPB), (unsigned)splits);
+    if (repl && peps) k_force_bundle1<NT, NRING, true, true, UMASS><<<grid, NT, 0, st>>>(A, group);
+    else if (repl) k_force_bundle1<NT, NRING, true, false, UMASS><<<grid, NT, 0, st>>>(A, group);
+    else if (peps) k_force_bundle1<NT, NRING, false, true, UMASS><<<grid, NT, 0, st>>>(A, group);
+    else k_force_bundle1<NT, NRING, false, false, UMASS><<<grid, NT, 0, st>>>(A, group);
+    return cudaGetLastError();
+}
+
+// one ray per lane (one tile per split): one-warp blocks while a tile's rays fit
+// one, else four warps, which share the staging of the tile
+cudaError_t dispatch_lanes(const ForceArgs &A, const ForceShape &sh, bool umass, cudaStream_t st)
+{
+    const int group = 2 * sh.NT;
+    const bool one = A.n / sh.R <= 32 / sh.R;
+    if (sh.R == 5) {
+        if (one) return umass ? go_lanes<32, 4, true>(A, group, sh.splits, st) : go_lanes<32, 4, false>(A, group, sh.splits, st);
+        return umass ? go_lanes<128, 4, true>(A, group, sh.splits, st) : go_lanes<128, 4, false>(A, group, sh.splits, st);
+    }
+    if (sh.R != 9) return cudaErrorInvalidConfiguration;
+    if (one) return umass ? go_lanes<32, 8, true>(A, group, sh.splits, st) : go_lanes<32, 8, false>(A, group, sh.splits, st);
+    return umass ? go_lanes<128, 8, true>(A, group, sh.splits, st) : go_lanes<128, 8, false>(A, group, sh.splits, st);
+}
+
 // rings of 4 (R = 5) or 8 (R = 9): grid.x counts blocks of 2 NT bundles,
 // grid.y the splits (a multiple of sh.cl).  With occ set nothing is launched:
 // *occ receives the kernel's resident blocks per SM.

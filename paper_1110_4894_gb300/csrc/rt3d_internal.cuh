@@ -269,6 +269,7 @@ struct ForceShape {
     int umass;    // packed kernel without per-particle masses (uniform-mass field)
     int cl = 1;   // thread-block cluster size along the splits: the cluster adds its
                   // CTAs' partials in distributed shared memory, one partial per cluster
+    int lanes = 0;  // variant 5: one ray per lane (k_force_bundle1), one tile per split
 };
 // split partials a shape leaves for the integrator stage
 inline int partial_splits(const ForceShape &sh) { return sh.splits / sh.cl; }
