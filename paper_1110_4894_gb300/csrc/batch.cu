@@ -190,9 +190,13 @@ __device__ __noinline__ void batch_grid_item(const BatchCone &C, int rb, int RB,
 template <int P, int NT, int MODE>
 __global__ void __launch_bounds__(NT, MODE == 5 ? 6 : 1) k_batch_run(BatchArgs B)
 {
-    __shared__ float4 s_a[kTile];
-    __shared__ float4 s_b[kTile];
-    __shared__ float2 s_e[kTile];
+    // a tile's records, or a prism item's sums: 10 kCorners doubles per group of
+    // lanes, kPrismLanes lanes at most
+    __shared__ float4 s_ab[2 * kTile + kTile / 2];
+    float4 *s_a = s_ab, *s_b = s_ab + kTile;
+    float2 *s_e = reinterpret_cast<float2 *>(s_ab + 2 * kTile);
+    constexpr int kPrismLanes = NT < 128 ? NT : 128;
+    static_assert(sizeof(s_ab) >= kPrismLanes * 10 * sizeof(double), "prism sums must fit the tile");
     __shared__ float2 s_hl[MODE == 5 ? 2 * (5 * 3 + 4) * NT : 1];
     __shared__ unsigned s_it;
     const int64_t nthreads = (int64_t)gridDim.x * NT;
@@ -213,9 +217,15 @@ __global__ void __launch_bounds__(NT, MODE == 5 ? 6 : 1) k_batch_run(BatchArgs B
             const int4 item = B.items[it];
             const BatchCone &C = B.cones[item.x];
             if (!cone_active(C, step)) continue;  // uniform across the block
-            if (item.z < 0) {  // the prism records of NT bundles (FP64)
-                const int64_t b = (int64_t)item.y * NT + threadIdx.x;
-                if (b < C.rs.n_b) bundle_prism(C.f, C.rs, g, b, C.prism);
+            if (item.z < 0) {  // the prism records of NT bundles (FP64), eight lanes to a bundle
+                if (threadIdx.x < kPrismLanes) {
+                    const int k = threadIdx.x / kCorners;
+                    double *s_q = reinterpret_cast<double *>(s_ab) + k * 10 * kCorners;
+                    for (int q = k; q < NT; q += kPrismLanes / kCorners) {
+                        const int64_t b = (int64_t)item.y * NT + q;
+                        bundle_prism(C.f, C.rs, g, b < C.rs.n_b ? b : -1, C.prism, s_q);
+                    }
+                }
                 continue;
             }
             if (item.w == 1) {  // a grid cone: App. B evaluation of one ray block (one split)

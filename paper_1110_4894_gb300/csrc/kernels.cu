@@ -69,11 +69,15 @@ cudaError_t launch_init(const TraceParams &tp, const DevField &f, const double *
 // integrator stage (Eq. geodesiceqn with the App. A symbols, classical RK4,
 // termination on x3 with linear interpolation: Sec. 3.4)
 // ---------------------------------------------------------------------------
-// A block of 256 threads serves 64 rays: first every thread reduces one
-// output of one ray's split partials (four threads per ray, which keeps four
-// times more loads in flight), then one thread per ray runs
-// the FP64 stage update with whole warps active.
-constexpr int kStageRays = 64;
+// Rays with many split partials: a block of four warps serves 32 rays.  Each
+// warp adds up one output of its rays, a serial double-float sum in split order
+// (reduce_step), then one warp runs the FP64 stage update of the 32 rays.  The
+// sum is a chain of thousands of steps in few warps where few bundles meet many
+// particles (4096 splits of 640 rays: 281 us a stage while its loads waited for
+// one another), so kAhead rows of partials are kept in flight in registers (84
+// us).
+constexpr int kStageRays = 32, kStageThreads = 4 * kStageRays;
+constexpr int kRows = 16, kAhead = 64;  // rows per load group, rows in flight
 // from this many rays on (four blocks of 256 per SM), one ray per thread
 // still gives every SM several blocks
 static int64_t stage_wide_rays() { return (int64_t)device_sm_count() * 4 * 256; }
@@ -91,52 +95,76 @@ int device_sm_count()
 }
 
 // the bundles' prism records of this stage (mean-subtracted boxes), read by
-// every ray of the bundle in k_stage
-__global__ void k_prism(TraceParams tp, DevField f, RayState rs, int step, int stage, const unsigned long long *cnt,
-                        double *__restrict__ prism)
+// every ray of the bundle in k_stage: one warp per block, four bundles of eight
+// lanes, so that few bundles still use the FP64 lanes of many SMs
+constexpr int kPrismBundles = 32 / kCorners;
+__global__ void __launch_bounds__(32) k_prism(TraceParams tp, DevField f, RayState rs, int step, int stage,
+                                              const unsigned long long *cnt, double *__restrict__ prism)
 {
+    __shared__ double s_q[kPrismBundles][10 * kCorners];
     if (step >= tp.n_steps && cnt[(step - 1) & 1] == 0ull) return;  // every ray is across
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= rs.n_b) return;
-    bundle_prism(f, rs, step * 4 + stage, b, prism);
+    const int k = threadIdx.x / kCorners;
+    const int64_t b = (int64_t)blockIdx.x * kPrismBundles + k;
+    bundle_prism(f, rs, step * 4 + stage, b < rs.n_b ? b : -1, prism, s_q[k]);
 }
 
 cudaError_t launch_prism(const TraceParams &tp, const DevField &f, RayState rs, int step, int stage,
                          const unsigned long long *d_counters, double *d_prism, cudaStream_t st)
 {
-    const int64_t blocks = (rs.n_b + 127) / 128;
-    k_prism<<<(unsigned)(blocks > 0 ? blocks : 1), 128, 0, st>>>(tp, f, rs, step, stage, d_counters, d_prism);
+    const int64_t blocks = (rs.n_b + kPrismBundles - 1) / kPrismBundles;
+    k_prism<<<(unsigned)(blocks > 0 ? blocks : 1), 32, 0, st>>>(tp, f, rs, step, stage, d_counters, d_prism);
     return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(256) k_stage(TraceParams tp, DevField f, RayState rs, int S, int fp64,
-                                              double mfac, const void *__restrict__ partials,
-                                              const double *__restrict__ dlam,
-                                              const double *__restrict__ misc, int step, int stage,
-                                              unsigned long long *cnt, const double *__restrict__ prism)
+__global__ void __launch_bounds__(kStageThreads) k_stage(TraceParams tp, DevField f, RayState rs, int S, int fp64,
+                                                        double mfac, const float2 *__restrict__ partials,
+                                                        const double *__restrict__ dlam,
+                                                        const double *__restrict__ misc, int step, int stage,
+                                                        unsigned long long *cnt, const double *__restrict__ prism)
 {
     if (stage == 0 && blockIdx.x == 0 && threadIdx.x == 0) cnt[step & 1] = 0ull;
     if (step >= tp.n_steps && cnt[(step - 1) & 1] == 0ull) return;  // every ray is across
     __shared__ double s_acc[kStageRays][4];
-    __shared__ unsigned s_active;
-    if (threadIdx.x == 0) s_active = 0;
-    const int64_t r0 = (int64_t)blockIdx.x * kStageRays;
-    {
-        const int local = threadIdx.x >> 2, o = threadIdx.x & 3;
-        const int64_t i = r0 + local;
-        if (i < rs.n_rays)
-            s_acc[local][o] = fp64 ? reduce_partials_fp64((const double *)partials, S, rs.n_rays, i, o)
-                                   : reduce_partials_mixed((const float2 *)partials, S, rs.n_rays, i, o);
+    const int o = threadIdx.x / kStageRays, lane = threadIdx.x % kStageRays;
+    const int64_t i = (int64_t)blockIdx.x * kStageRays + lane;
+    if (i < rs.n_rays) {
+        constexpr int G = kAhead / kRows;
+        const float2 *src = partials + (int64_t)o * rs.n_rays + i;
+        const int64_t pitch = 4 * rs.n_rays;
+        float2 buf[G][kRows];
+        // (rows past the last split are zeros, which leave the sum as it is)
+        const auto load = [&](int g, int s0) {
+#pragma unroll
+            for (int r = 0; r < kRows; ++r, src += pitch)
+                buf[g][r] = s0 + r < S ? __ldg(src) : make_float2(0.0f, 0.0f);
+        };
+#pragma unroll
+        for (int g = 0; g < G; ++g) load(g, g * kRows);
+        float hi = 0.0f, lo = 0.0f;
+        double acc = 0.0;
+        for (int s0 = 0; s0 < S; s0 += kAhead) {
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                if (s0 + g * kRows >= S) break;
+                if (fp64) {
+#pragma unroll
+                    for (int r = 0; r < kRows; ++r)
+                        acc += __hiloint2double(__float_as_int(buf[g][r].y), __float_as_int(buf[g][r].x));
+                } else {
+#pragma unroll
+                    for (int r = 0; r < kRows; ++r) reduce_step(hi, lo, buf[g][r]);
+                }
+                load(g, s0 + kAhead + g * kRows);
+            }
+        }
+        s_acc[lane][o] = fp64 ? acc : (double)hi + (double)lo;
     }
     __syncthreads();
-    if (threadIdx.x < kStageRays) {
-        const int64_t i = r0 + threadIdx.x;
-        if (i < rs.n_rays && stage_ray(tp, f, rs, S, fp64 != 0, mfac, partials, dlam, misc[0], step, stage, cnt, i,
-                                       s_acc[threadIdx.x], prism))
-            atomicAdd(&s_active, 1u);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && s_active) atomicAdd(&cnt[2], (unsigned long long)s_active);
+    if (threadIdx.x >= kStageRays) return;
+    const bool act = i < rs.n_rays && stage_ray(tp, f, rs, S, fp64 != 0, mfac, partials, dlam, misc[0], step, stage, cnt, i,
+                                                s_acc[lane], prism);
+    const unsigned m = __ballot_sync(0xffffffffu, act);
+    if (lane == 0 && m) atomicAdd(&cnt[2], (unsigned long long)__popc(m));
 }
 
 // One ray per thread, its four outputs reduced by the same thread: for few
@@ -175,13 +203,17 @@ cudaError_t launch_stage(const TraceParams &tp, const DevField &f, RayState rs, 
     const int S = partial_splits(sh);
     const double mfac = partial_mass_factor(f, sh);
     if (S <= 8 || rs.n_rays >= stage_wide_rays()) {
-        const int64_t blocks = (rs.n_rays + 255) / 256;
-        k_stage_wide<<<(unsigned)blocks, 256, 0, st>>>(tp, f, rs, S, fp64 ? 1 : 0, mfac, d_partials, d_dlam, d_misc,
-                                                       step, stage, d_counters, d_prism);
+        // the two FP64 lanes of an SM serve all its warps: few rays go one warp
+        // per block, to as many SMs as there are
+        int nt = 256;
+        while (nt > 32 && rs.n_rays < 2 * (int64_t)device_sm_count() * nt) nt /= 2;
+        const int64_t blocks = (rs.n_rays + nt - 1) / nt;
+        k_stage_wide<<<(unsigned)blocks, nt, 0, st>>>(tp, f, rs, S, fp64 ? 1 : 0, mfac, d_partials, d_dlam, d_misc,
+                                                      step, stage, d_counters, d_prism);
     } else {
         const int64_t blocks = (rs.n_rays + kStageRays - 1) / kStageRays;
-        k_stage<<<(unsigned)blocks, 256, 0, st>>>(tp, f, rs, S, fp64 ? 1 : 0, mfac, d_partials, d_dlam, d_misc, step,
-                                                 stage, d_counters, d_prism);
+        k_stage<<<(unsigned)blocks, kStageThreads, 0, st>>>(tp, f, rs, S, fp64 ? 1 : 0, mfac, (const float2 *)d_partials,
+                                                            d_dlam, d_misc, step, stage, d_counters, d_prism);
     }
     return cudaGetLastError();
 }

@@ -127,6 +127,28 @@ __device__ __forceinline__ void prism_field(const T lo[3], const T hi[3], const 
     out[3] = gz;
 }
 
+// One corner's terms, unsigned: F and its first derivatives as prism_corner,
+// the pure second derivatives tx, ty, tz, then the mixed xy, xz, yz
+__device__ __forceinline__ void prism_corner_hess(double x, double y, double z, double v[10])
+{
+    const double xx = x * x, yy = y * y, zz = z * z;
+    const double rho = sqrt(xx + yy + zz);
+    const double lx = prism_log(x, rho, yy + zz), ly = prism_log(y, rho, xx + zz), lz = prism_log(z, rho, xx + yy);
+    const double tx = (x != 0.0) ? atan(y * z / (x * rho)) : 0.0;
+    const double ty = (y != 0.0) ? atan(z * x / (y * rho)) : 0.0;
+    const double tz = (z != 0.0) ? atan(x * y / (z * rho)) : 0.0;
+    v[0] = x * y * lz + y * z * lx + z * x * ly - 0.5 * (xx * tx + yy * ty + zz * tz);
+    v[1] = y * lz + z * ly - x * tx;
+    v[2] = z * lx + x * lz - y * ty;
+    v[3] = x * ly + y * lx - z * tz;
+    v[4] = tx;
+    v[5] = ty;
+    v[6] = tz;
+    v[7] = lz;
+    v[8] = ly;
+    v[9] = lx;
+}
+
 // As prism_field, plus the Hessian d2I/dp_i dp_j (h = xx, xy, xz, yy, yz,
 // zz) from the same logarithms and arctangents: for the corner function,
 // d2F/dx2 = -atan(yz / (x rho)) and d2F/dx dy = log(z + rho) (cyclically).

@@ -1,0 +1,31 @@
+"""The integrator stage's sum of split partials around its groups of 16 and 64
+rows: the same trace with any number of splits.  The partials are compensated
+pairs (FP32 pair sums) or FP64 sums, so regrouping moves the field by 2^-45 or
+less, except the potential, an FP32 sum per split (1e-6 of itself, which enters
+the geodesics at 1e-11 of the path): mu stays within 1e-9 of its largest
+value, on this weak field."""
+import numpy as np
+import pytest
+
+import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+@pytest.mark.parametrize("bundles", [1, 7, 40])
+def test_any_number_of_splits(precision, bundles):
+    import paper_1110_4894_gb300 as P
+    n = 256 * 130
+    g = inputs.rng(inputs.BASE_SEED + 130)
+    pos = inputs.quantize(np.array([0.0, 0.0, 1000.0]) + 0.5 * g.normal(size=(n, 3)))
+    theta = np.array([3e-4, -2e-4]) + 2e-4 * g.normal(size=(bundles, 2))
+    res = []
+    for splits in (8, 9, 15, 16, 17, 63, 64, 65, 128, 130):
+        ctx = P.Context(0, precision=P.FP64 if precision == "fp64" else P.MIXED, splits=splits)
+        ctx.set_cosmology(0.3, 0.7, 0.7)
+        ctx.load_particles(0, pos, 1e9, 0.05)
+        res.append(ctx.trace(0, 0.5, theta, n_ring=4, theta_r=5e-6, n_steps=6)["mu"])
+        ctx.close()
+    for r in res[1:]:
+        assert np.max(np.abs(r - res[0])) <= 1e-9 * np.max(np.abs(res[0]))
