@@ -94,38 +94,91 @@ __global__ void k_fill_mass(int n, const unsigned long long *__restrict__ q, con
     }
 }
 
-// kernel f on the padded grid, indexed by node displacement
-// (k < n: +k, k > n: k - 2n, k = n: unused, zero)
-__global__ void k_fill_kernel(int n, int f, double h, double eps2, double *__restrict__ buf)
+// the convolution kernels for node displacements 0..n-1 per axis (phi, then
+// grad phi where nf = 4 or its x1 component where nf = 2), kernel-major: each
+// square root and division (some forty FP64 operations) once, for all the
+// octants and kernels that share it
+__global__ void k_kernel_octant(int n, int nf, double h, double eps2, double *__restrict__ oct)
+{
+    const int64_t m = (int64_t)n * n * n;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+        const int k[3] = {(int)(i / ((int64_t)n * n)), (int)((i / n) % n), (int)(i % n)};
+        double d[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) d[c] = (double)k[c] * h;
+        const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2] + eps2;
+        const double inv = r2 > 0.0 ? 1.0 / sqrt(r2) : 0.0;
+        oct[i] = -kMuG * inv;
+        for (int f = 1; f < nf; ++f) oct[f * m + i] = kMuG * d[f - 1] * inv * inv * inv;
+    }
+}
+
+// kernel f on the padded (P = 2n)^3 grid from its octant, indexed by node
+// displacement (k < n: +k, k > n: k - 2n, k = n: unused, zero); a gradient
+// kernel is odd along its axis
+__global__ void k_unfold(int n, int f, const double *__restrict__ oct, double *__restrict__ buf)
 {
     const int P = 2 * n;
     const int64_t m = (int64_t)P * P * P;
+    oct += f * ((int64_t)n * n * n);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
         const int k[3] = {(int)(i / ((int64_t)P * P)), (int)((i / P) % P), (int)(i % P)};
-        double d[3];
-        bool ok = true;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            ok = ok && k[c] != n;
-            d[c] = (double)(k[c] < n ? k[c] : k[c] - P) * h;
-        }
-        const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2] + eps2;
         double v = 0.0;
-        if (ok && r2 > 0.0) {
-            const double inv = 1.0 / sqrt(r2);
-            v = f == 0 ? -kMuG * inv : kMuG * d[f - 1] * inv * inv * inv;
+        if (k[0] != n && k[1] != n && k[2] != n) {
+            const int q[3] = {k[0] < n ? k[0] : P - k[0], k[1] < n ? k[1] : P - k[1], k[2] < n ? k[2] : P - k[2]};
+            v = oct[((int64_t)q[0] * n + q[1]) * n + q[2]];
+            if (f > 0 && k[f - 1] > n) v = -v;
         }
         buf[i] = v;
     }
+}
+
+__device__ __forceinline__ cufftDoubleComplex cmul_scaled(cufftDoubleComplex x, cufftDoubleComplex y, double scale)
+{
+    return make_cuDoubleComplex((x.x * y.x - x.y * y.y) * scale, (x.x * y.y + x.y * y.x) * scale);
 }
 
 // out = a b scale (out may be b)
 __global__ void k_cmul(int64_t m, const cufftDoubleComplex *__restrict__ a, const cufftDoubleComplex *b,
                        cufftDoubleComplex *out, double scale)
 {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = cmul_scaled(a[i], b[i], scale);
+}
+
+// The grid is a cube, so the x2 and x3 gradient kernels are the x1 kernel with
+// two axes exchanged, and so are their spectra (half spectra [k1][k2][k3 <= n]):
+// out = a b' scale with b'(k1, k2, k3) = b(k2, k1, k3), or b(k3, k2, k1), where
+// the x1 kernel is even along x3, b(., ., P - k) = b(., ., k).  That saves two
+// of the five forward transforms.
+__global__ void k_cmul_x2(int n, const cufftDoubleComplex *__restrict__ a, const cufftDoubleComplex *__restrict__ b,
+                          cufftDoubleComplex *__restrict__ out, double scale)
+{
+    const int P = 2 * n, H = n + 1;
+    const int64_t m = (int64_t)P * P * H;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        const cufftDoubleComplex x = a[i], y = b[i];
-        out[i] = make_cuDoubleComplex((x.x * y.x - x.y * y.y) * scale, (x.x * y.y + x.y * y.x) * scale);
+        const int64_t k3 = i % H, k2 = (i / H) % P, k1 = i / ((int64_t)P * H);
+        out[i] = cmul_scaled(a[i], b[(k2 * P + k1) * H + k3], scale);
+    }
+}
+
+constexpr int kCmulTile = 16;  // k1 x k3 tile, transposed through shared memory
+__global__ void __launch_bounds__(kCmulTile *kCmulTile) k_cmul_x3(int n, const cufftDoubleComplex *__restrict__ a,
+                                                                const cufftDoubleComplex *__restrict__ b,
+                                                                cufftDoubleComplex *__restrict__ out, double scale)
+{
+    __shared__ cufftDoubleComplex s[kCmulTile][kCmulTile + 1];
+    const int P = 2 * n, H = n + 1;
+    const int c0 = blockIdx.x * kCmulTile, a0 = blockIdx.y * kCmulTile, k2 = blockIdx.z;
+    const int x = threadIdx.x, y = threadIdx.y;
+    if (c0 + y < H && a0 + x < P) {
+        const int k = a0 + x <= n ? a0 + x : P - (a0 + x);
+        s[y][x] = b[((int64_t)(c0 + y) * P + k2) * H + k];
+    }
+    __syncthreads();
+    if (c0 + x < H && a0 + y < P) {
+        const int64_t i = ((int64_t)(a0 + y) * P + k2) * H + c0 + x;
+        out[i] = cmul_scaled(a[i], s[x][y], scale);
     }
 }
 
@@ -144,13 +197,10 @@ __global__ void k_extract(int n, const double *__restrict__ buf, double *__restr
 // The elimination factors depend on n only and are shared by all lines.
 __global__ void k_spline_lines(int n, int64_t lines, const double *__restrict__ val, double *__restrict__ y2)
 {
-    __shared__ double s_den[kMaxGridN];
+    __shared__ double s_inv[kMaxGridN];  // 1 / the elimination's pivots
     if (threadIdx.x == 0) {
         double cp = 0.0;
-        for (int i = 1; i <= n - 2; ++i) {
-            s_den[i] = 4.0 - cp;
-            cp = 1.0 / s_den[i];
-        }
+        for (int i = 1; i <= n - 2; ++i) s_inv[i] = cp = 1.0 / (4.0 - cp);
     }
     __syncthreads();
     const int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -162,10 +212,10 @@ __global__ void k_spline_lines(int n, int64_t lines, const double *__restrict__ 
     if (n < 3) return;
     double dp = 0.0;
     for (int i = 1; i <= n - 2; ++i) {
-        dp = (6.0 * (y[i + 1] - 2.0 * y[i] + y[i - 1]) - dp) / s_den[i];
+        dp = (6.0 * (y[i + 1] - 2.0 * y[i] + y[i - 1]) - dp) * s_inv[i];
         z[i] = dp;
     }
-    for (int i = n - 3; i >= 1; --i) z[i] = z[i] - z[i + 1] / s_den[i];
+    for (int i = n - 3; i >= 1; --i) z[i] = z[i] - z[i + 1] * s_inv[i];
 }
 
 // node table: per node the four values, then the four x3-spline second
@@ -385,7 +435,7 @@ cudaError_t launch_grid_eval(const GridDev &g, const double *px, const double *p
 // stage, a trace was an evaluation and an update kernel per stage with the
 // state, the field and their launches between them: 11.5 + 5.9 us for 20,480
 // rays and a 128^3 grid; grid and trace of 500 steps together 75.6 -> 36.4 ms
-// (the grid is 20 ms of both).  What is left is each stage's
+// (the grid was 20 ms of both).  What is left is each stage's
 // FP64 (about 150 operations per ray on two lanes per SM) behind the latency of
 // its node gather.  A bundle whose rays are all across stops: results are
 // taken at the crossing, and the stages after it only served other bundles.
@@ -508,18 +558,25 @@ static unsigned blocks_for(int64_t m)
 namespace {
 // Device state for building grids of one shape (n nodes per side, spacing h,
 // softening eps): FFT buffers and plans, node-mass and value temporaries, and
-// (when cache_kernels) the four kernel spectra, which depend on the shape
-// only and so serve every cube of a replicated box.  Freed on every exit.
+// (keep: where they fit) the spectra of the phi and x1 kernels, which give all
+// four, depend on the shape only and so serve every cube of a replicated box.
+// Freed on every exit.
+//
+// A 3D transform is one over the (x2, x3) planes and one along x1: the node
+// masses fill, and the node values need, only the first half of the planes, so
+// the plane transforms of the other half are left out (the FP64 of the
+// transforms bounds the build; 128^3 nodes: 15.8 -> 9.1 ms of them, and 3.4 ->
+// 0.3 ms for the kernels they transform).
 struct Builder {
     int n = 0;
     double h = 0.0, eps2 = 0.0;
-    bool cache = false, have_k = false;
+    bool keep = false, have_k = false;
     double *pos = nullptr, *mass = nullptr, *buf = nullptr, *val = nullptr, *y2 = nullptr;
     int64_t cap = 0;
     unsigned long long *q = nullptr, *total = nullptr;
     cufftDoubleComplex *fm = nullptr, *fk = nullptr, *kspec = nullptr;
-    cufftHandle r2c = 0, c2r = 0;
-    bool have_r2c = false, have_c2r = false;
+    cufftHandle r2c = 0, c2r = 0, c2c = 0;  // half the planes, both ways; along x1
+    bool have_r2c = false, have_c2r = false, have_c2c = false;
     std::string *err = nullptr;
     ~Builder()
     {
@@ -535,6 +592,7 @@ struct Builder {
         cudaFree(kspec);
         if (have_r2c) cufftDestroy(r2c);
         if (have_c2r) cufftDestroy(c2r);
+        if (have_c2c) cufftDestroy(c2c);
     }
     int cuda_fail(cudaError_t e, const char *what)
     {
@@ -563,16 +621,13 @@ struct Builder {
         if (r_ != CUFFT_SUCCESS) return B.fft_fail(r_, what); \
     } while (0)
 
-static int builder_init(Builder &B, int n, double h, double soft, bool cache_kernels, cudaStream_t st,
-                        std::string &err)
+static int builder_init(Builder &B, int n, double h, double soft, cudaStream_t st, std::string &err)
 {
     B.n = n;
     B.h = h;
     B.eps2 = soft * soft;
     B.err = &err;
     const int P = 2 * n;
-    // the four kernel spectra stay resident only where they are small
-    B.cache = cache_kernels && 4 * B.Pc() * (int64_t)sizeof(cufftDoubleComplex) <= ((int64_t)8 << 30);
     GCK(cudaMalloc(&B.q, sizeof(unsigned long long) * (size_t)B.n3()), "grid node buffer");
     GCK(cudaMalloc(&B.total, sizeof(unsigned long long)), "grid total");
     GCK(cudaMalloc(&B.buf, sizeof(double) * (size_t)B.P3()), "grid FFT buffer");
@@ -580,13 +635,24 @@ static int builder_init(Builder &B, int n, double h, double soft, bool cache_ker
     GCK(cudaMalloc(&B.fk, sizeof(cufftDoubleComplex) * (size_t)B.Pc()), "grid FFT buffer");
     GCK(cudaMalloc(&B.val, sizeof(double) * 4 * (size_t)B.n3()), "grid values");
     GCK(cudaMalloc(&B.y2, sizeof(double) * 4 * (size_t)B.n3()), "grid spline table");
-    if (B.cache) GCK(cudaMalloc(&B.kspec, sizeof(cufftDoubleComplex) * 4 * (size_t)B.Pc()), "grid kernel spectra");
-    FCK(cufftPlan3d(&B.r2c, P, P, P, CUFFT_D2Z), "cufftPlan3d D2Z");
+    int plane[2] = {P, P}, half[2] = {P, n + 1}, line[1] = {P};
+    const int pd = P * P, pc = P * (n + 1);
+    FCK(cufftPlanMany(&B.r2c, 2, plane, plane, 1, pd, half, 1, pc, CUFFT_D2Z, n), "cufftPlanMany D2Z");
     B.have_r2c = true;
-    FCK(cufftPlan3d(&B.c2r, P, P, P, CUFFT_Z2D), "cufftPlan3d Z2D");
+    FCK(cufftPlanMany(&B.c2r, 2, plane, half, 1, pc, plane, 1, pd, CUFFT_Z2D, n), "cufftPlanMany Z2D");
     B.have_c2r = true;
+    FCK(cufftPlanMany(&B.c2c, 1, line, line, pc, 1, line, pc, 1, CUFFT_Z2Z, pc), "cufftPlanMany Z2Z");
+    B.have_c2c = true;
     FCK(cufftSetStream(B.r2c, st), "cufftSetStream");
     FCK(cufftSetStream(B.c2r, st), "cufftSetStream");
+    FCK(cufftSetStream(B.c2c, st), "cufftSetStream");
+    // the two kernel spectra stay resident where they are small and fit
+    B.keep = 2 * B.Pc() * (int64_t)sizeof(cufftDoubleComplex) <= ((int64_t)8 << 30);
+    if (B.keep && cudaMalloc(&B.kspec, sizeof(cufftDoubleComplex) * 2 * (size_t)B.Pc()) != cudaSuccess) {
+        cudaGetLastError();
+        B.kspec = nullptr;
+        B.keep = false;
+    }
     return RT3D_OK;
 }
 
@@ -626,21 +692,46 @@ static int builder_run(Builder &B, int64_t np, const double *pos, const double *
     GCK(cudaGetLastError(), "k_sum_q");
     k_fill_mass<<<blocks_for(P3), 256, 0, st>>>(n, B.q, B.total, qinv, mean_subtract, B.buf);
     GCK(cudaGetLastError(), "k_fill_mass");
-    FCK(cufftExecD2Z(B.r2c, B.buf, B.fm), "cufftExecD2Z");
+    const int P = 2 * n;
+    const int64_t half_d = P3 / 2, half_c = Pc / 2;
+    FCK(cufftExecD2Z(B.r2c, B.buf, B.fm), "cufftExecD2Z");  // the masses' planes; the others are zero
+    GCK(cudaMemsetAsync(B.fm + half_c, 0, sizeof(cufftDoubleComplex) * (size_t)half_c, st), "memset");
+    FCK(cufftExecZ2Z(B.c2c, B.fm, B.fm, CUFFT_FORWARD), "cufftExecZ2Z");
+    const auto kernel_spectrum = [&](int f, cufftDoubleComplex *ks) -> int {
+        k_unfold<<<blocks_for(P3), 256, 0, st>>>(n, f, B.y2, B.buf);
+        GCK(cudaGetLastError(), "k_unfold");
+        FCK(cufftExecD2Z(B.r2c, B.buf, ks), "cufftExecD2Z");
+        FCK(cufftExecD2Z(B.r2c, B.buf + half_d, ks + half_c), "cufftExecD2Z");
+        FCK(cufftExecZ2Z(B.c2c, ks, ks, CUFFT_FORWARD), "cufftExecZ2Z");
+        return RT3D_OK;
+    };
+    if (!B.have_k) {  // (the octants wait where the splines will be)
+        k_kernel_octant<<<blocks_for(n3), 256, 0, st>>>(n, B.keep ? 2 : 4, B.h, B.eps2, B.y2);
+        GCK(cudaGetLastError(), "k_kernel_octant");
+        for (int f = 0; f < 2 && B.keep; ++f)
+            if (const int rc = kernel_spectrum(f, B.kspec + f * Pc)) return rc;
+        B.have_k = B.keep;
+    }
+    const double scale = 1.0 / (double)P3;
     for (int f = 0; f < 4; ++f) {
-        cufftDoubleComplex *ks = B.cache ? B.kspec + f * Pc : B.fk;
-        if (!B.cache || !B.have_k) {
-            k_fill_kernel<<<blocks_for(P3), 256, 0, st>>>(n, f, B.h, B.eps2, B.buf);
-            GCK(cudaGetLastError(), "k_fill_kernel");
-            FCK(cufftExecD2Z(B.r2c, B.buf, ks), "cufftExecD2Z");
+        if (!B.keep) {
+            if (const int rc = kernel_spectrum(f, B.fk)) return rc;
+            k_cmul<<<blocks_for(Pc), 256, 0, st>>>(Pc, B.fm, B.fk, B.fk, scale);
+        } else if (f < 2) {
+            k_cmul<<<blocks_for(Pc), 256, 0, st>>>(Pc, B.fm, B.kspec + f * Pc, B.fk, scale);
+        } else if (f == 2) {
+            k_cmul_x2<<<blocks_for(Pc), 256, 0, st>>>(n, B.fm, B.kspec + Pc, B.fk, scale);
+        } else {
+            const dim3 tiles((unsigned)((n + kCmulTile) / kCmulTile), (unsigned)((P + kCmulTile - 1) / kCmulTile),
+                             (unsigned)P);
+            k_cmul_x3<<<tiles, dim3(kCmulTile, kCmulTile), 0, st>>>(n, B.fm, B.kspec + Pc, B.fk, scale);
         }
-        k_cmul<<<blocks_for(Pc), 256, 0, st>>>(Pc, B.fm, ks, B.fk, 1.0 / (double)P3);
         GCK(cudaGetLastError(), "k_cmul");
+        FCK(cufftExecZ2Z(B.c2c, B.fk, B.fk, CUFFT_INVERSE), "cufftExecZ2Z");
         FCK(cufftExecZ2D(B.c2r, B.fk, B.buf), "cufftExecZ2D");
         k_extract<<<blocks_for(n3), 256, 0, st>>>(n, B.buf, B.val + f * n3);
         GCK(cudaGetLastError(), "k_extract");
     }
-    B.have_k = B.cache;
     const int64_t lines = 4 * (int64_t)n * n;
     k_spline_lines<<<(unsigned)((lines + 127) / 128), 128, 0, st>>>(n, lines, B.val, B.y2);
     GCK(cudaGetLastError(), "k_spline_lines");
@@ -653,7 +744,7 @@ int grid_build(GridDev &g, int64_t np, const double *pos, const double *mass, do
                bool fp64, cudaStream_t st, std::string &err)
 {
     Builder B;
-    int rc = builder_init(B, g.n, g.h, soft, false, st, err);
+    int rc = builder_init(B, g.n, g.h, soft, st, err);
     if (rc != RT3D_OK) return rc;
     if (fp64)
         GCK(cudaMalloc(&g.tab, sizeof(double) * kGridRec * (size_t)B.n3()), "grid node table");
@@ -722,7 +813,7 @@ int grid_build_box(GridDev &g, int64_t np, const double *pos, const double *mass
             }
     }
     Builder B;
-    int rc = builder_init(B, g.n, g.h, soft, true, st, err);
+    int rc = builder_init(B, g.n, g.h, soft, st, err);
     if (rc != RT3D_OK) return rc;
     const size_t stride = kGridRec * (size_t)B.n3();
     if (fp64)
