@@ -916,6 +916,11 @@ __device__ __forceinline__ void bundle2x_block_sum(const DevField &f, const doub
                     float2 R2 = __ffma2_rn(DZ, DZ, E2);
                     R2 = __ffma2_rn(DY, DY, R2);
                     R2 = __ffma2_rn(DX, DX, R2);
+                    // every ray's 1 / r first, so that the reciprocal square roots
+                    // of all of them are under way before the first is used
+                    // (0.7 % faster for rings of 4, 2 % for rings of 8; starting the
+                    // next particle's in this one's place is 10 % slower)
+                    float2 w[NR];
 #pragma unroll
                     for (int g = 0; g < NR; ++g) {
                         float2 s2 = R2;
@@ -925,14 +930,17 @@ __device__ __forceinline__ void bundle2x_block_sum(const DevField &f, const doub
                             t = __ffma2_rn(fx[g - 1], DX, t);
                             s2 = __fadd2_rn(R2, t);
                         }
-                        const float2 w = make_float2(rsqrt_mufu(s2.x), rsqrt_mufu(s2.y));
-                        const float2 u = __fmul2_rn(w, w);
+                        w[g] = make_float2(rsqrt_mufu(s2.x), rsqrt_mufu(s2.y));
+                    }
+#pragma unroll
+                    for (int g = 0; g < NR; ++g) {
+                        const float2 u = __fmul2_rn(w[g], w[g]);
                         float2 m3;
                         if (UMASS) {
-                            if (g == 0) phi = __fadd2_rn(phi, w);
-                            m3 = __fmul2_rn(w, u);
+                            if (g == 0) phi = __fadd2_rn(phi, w[g]);
+                            m3 = __fmul2_rn(w[g], u);
                         } else {
-                            const float2 mw = __fmul2_rn(M2, w);
+                            const float2 mw = __fmul2_rn(M2, w[g]);
                             if (g == 0) phi = __fadd2_rn(phi, mw);
                             m3 = __fmul2_rn(mw, u);
                         }
