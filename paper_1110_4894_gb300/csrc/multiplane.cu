@@ -314,8 +314,12 @@ __global__ void __launch_bounds__(kMpNT) k_mp_deflect(MPArgs A)
 // 2 (1 + NRING) reciprocals.  Same outputs and layout as k_mp_deflect.
 constexpr int kMp2NT = 64;
 
-// (rings of 4 bounded for 8 blocks per SM, 128 registers; rings of 8, whose
-// accumulators need more, for 4)
+// Only the particles on the plane are staged (in their order), so that a plane
+// costs its own particles and not the whole replica's; what is left per plane is
+// the look at every particle.  524,288 particles, 4096 bundles to z = 0.5: 115.1
+// -> 69.1 ms for two planes per replica; one per replica takes 59.2.
+// (rings of 4 bounded for 8 blocks per SM, 128 registers, as fast as 7 and 5 %
+// faster than 6; rings of 8, whose accumulators need more, for 4)
 template <int NRING, bool REPL, bool PEPS, bool UMASS>
 __global__ void __launch_bounds__(kMp2NT, NRING <= 4 ? 8 : 4) k_mp_deflect2(MPArgs A)
 {
@@ -326,6 +330,7 @@ __global__ void __launch_bounds__(kMp2NT, NRING <= 4 ? 8 : 4) k_mp_deflect2(MPAr
     __shared__ float4 s_a[kTile + 1];  // + 1: the particle loop reads one record ahead
     __shared__ float4 s_b[kTile + 1];
     __shared__ float2 s_hl[2 * NQ * kMp2NT];  // (hi, lo) of output q for the pair (A, B)
+    __shared__ int s_cnt[kTile / 32];          // on-plane particles of each staging round and warp
     const DevField &f = A.f;
     const int tid = threadIdx.x;
     const int64_t b0 = (int64_t)blockIdx.x * 2 * kMp2NT;
@@ -372,25 +377,47 @@ __global__ void __launch_bounds__(kMp2NT, NRING <= 4 ? 8 : 4) k_mp_deflect2(MPAr
     const int64_t p1 = min(f.n, p0 + A.per_split);
     const float dlt = (float)f.delta;
     for (int64_t t0 = p0; t0 < p1; t0 += kTile) {
-        __syncthreads();
-        for (int qq = tid; qq < kTile; qq += kMp2NT) {
-            const int64_t pi = t0 + qq;
-            float x = -1e18f, y = -1e18f, m = 0.f, e = 0.f;
+        // Stage the tile's particles that are on the plane, in their order: a
+        // box's slab is one of `slices` of its replica, so most of a tile may
+        // be off it, and every record of the loop below costs the same.
+        constexpr int K = kTile / kMp2NT, NW = kMp2NT / 32;
+        const int lane = tid & 31, warp = tid >> 5;
+        float4 rec[K];  // x, y, m, eps^2
+        unsigned on[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int64_t pi = t0 + k * kMp2NT + tid;
+            bool in = false;
             if (pi < p1) {
                 const int4 pr = f.part[pi];
                 long long g[3] = {pr.x, pr.y, pr.z};
                 if (REPL) replica_q(f, P.rep, pr.x, pr.y, pr.z, g);
-                if (g[2] >= P.qlo && g[2] <= P.qhi) {
-                    ++n_on;
-                    x = -(float)(g[0] - ax) * dlt;
-                    y = -(float)(g[1] - ay) * dlt;
-                    m = __int_as_float(pr.w);
-                    e = PEPS ? f.eps2[pi] : f.eps2u;
-                }
+                in = g[2] >= P.qlo && g[2] <= P.qhi;
+                rec[k] = make_float4(-(float)(g[0] - ax) * dlt, -(float)(g[1] - ay) * dlt, __int_as_float(pr.w),
+                                   PEPS ? f.eps2[pi] : f.eps2u);
             }
-            s_a[qq] = make_float4(x, x, y, y);
-            s_b[qq] = make_float4(m, m, e, e);
+            on[k] = __ballot_sync(0xffffffffu, in);
         }
+        __syncthreads();  // every thread is done with the tile before
+        if (lane == 0)
+#pragma unroll
+            for (int k = 0; k < K; ++k) s_cnt[k * NW + warp] = __popc(on[k]);
+        __syncthreads();
+        int m = 0, at[K];
+#pragma unroll
+        for (int c = 0; c < K * NW; ++c) {
+            if (c % NW == warp) at[c / NW] = m;
+            m += s_cnt[c];
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (on[k] >> lane & 1u) {
+                const int q = at[k] + __popc(on[k] & ((1u << lane) - 1u));
+                s_a[q] = make_float4(rec[k].x, rec[k].x, rec[k].y, rec[k].y);
+                s_b[q] = make_float4(rec[k].z, rec[k].z, rec[k].w, rec[k].w);
+            }
+        if (tid == 0) n_on += m;
+        if (m == 0) continue;
         __syncthreads();
         float2 cx = make_float2(0.f, 0.f), cy = cx, gx[NRING], gy[NRING], gs[NRING];
 #pragma unroll
@@ -400,7 +427,7 @@ __global__ void __launch_bounds__(kMp2NT, NRING <= 4 ? 8 : 4) k_mp_deflect2(MPAr
         // current particle's arithmetic
         float4 a_nx = s_a[0], b_nx = s_b[0];
 #pragma unroll 1
-        for (int jj = 0; jj < kTile; ++jj) {
+        for (int jj = 0; jj < m; ++jj) {
             const float4 a = a_nx;
             const float4 b = b_nx;
             a_nx = s_a[jj + 1];
