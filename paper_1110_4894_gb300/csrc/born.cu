@@ -52,6 +52,47 @@ __global__ void k_born_points(DevField f, int64_t n_b, const double *__restrict_
     rep[q] = replica_of(f, xk);
 }
 
+// One staged tile's terms into a thread's R points, in chunks of kChunk merged
+// by TwoSum.  The kernel is bound by instruction issue (20 FP32 operations and a
+// reciprocal square root per pair at 88 % of the slots), so what can be saved
+// without another rounding is: half of A is summed (-3 / 2 and 1 instead of -3
+// and 2, all powers of two apart), and a thread whose points lie on one node
+// (FLAT: most are, node-major) forms dz once: 67.0 -> 60.1 ms for 2048 lines of
+// sight x 501 nodes x 100,000 particles.
+template <int R, bool PEPS, bool FLAT>
+__device__ __forceinline__ void hess_tile(const float4 *s_p, const float *s_e, float eps2u, const float (&rx)[R],
+                                          const float (&ry)[R], const float (&rz)[R], float (&hi)[R][3],
+                                          float (&lo)[R][3])
+{
+    for (int c0 = 0; c0 < kTile; c0 += kChunk) {
+        float ca[R][3];
+#pragma unroll
+        for (int k = 0; k < R; ++k) ca[k][0] = ca[k][1] = ca[k][2] = 0.0f;
+#pragma unroll 4
+        for (int jj = c0; jj < c0 + kChunk; ++jj) {
+            const float4 p = s_p[jj];
+            const float e2 = PEPS ? s_e[jj] : eps2u;
+            const float dz0 = rz[0] - p.z;
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                const float dx = rx[k] - p.x, dy = ry[k] - p.y, dz = FLAT ? dz0 : rz[k] - p.z;
+                const float dxx = dx * dx, dyy = dy * dy;
+                const float r2 = fmaf(dz, dz, dxx + dyy) + e2;
+                const float inv = rsqrt_mufu(r2);
+                const float i2 = inv * inv;
+                const float m3 = p.w * inv * i2, m5 = m3 * i2;
+                ca[k][0] += fmaf(-1.5f * (dxx + dyy), m5, m3);
+                ca[k][1] = fmaf(dyy - dxx, m5, ca[k][1]);
+                ca[k][2] = fmaf(dx * dy, m5, ca[k][2]);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < R; ++k)
+#pragma unroll
+            for (int o2 = 0; o2 < 3; ++o2) two_sum_into(hi[k][o2], lo[k][o2], ca[k][o2]);
+    }
+}
+
 // Hessian pair sum: for every point, sums over particles [p0, p1) of
 //   A = m (2 / r^3 - 3 (dx^2 + dy^2) / r^5),  B = m (dy^2 - dx^2) / r^5,
 //   C = m dx dy / r^5          (d = point - particle, r^2 = |d|^2 + eps^2)
@@ -95,6 +136,10 @@ __global__ void __launch_bounds__(NT) k_hess(ForceArgs A)
                 rx[k] = ry[k] = rz[k] = 5e18f;
             }
         }
+        bool flat = true;  // the points of one node share their x3
+#pragma unroll
+        for (int k = 1; k < R; ++k) flat = flat && rz[k] == rz[0];
+        flat = __syncthreads_and(flat) != 0;
         for (int64_t t0 = p0; t0 < p1; t0 += kTile) {
             __syncthreads();
             for (int q = tid; q < kTile; q += NT) {
@@ -113,32 +158,8 @@ __global__ void __launch_bounds__(NT) k_hess(ForceArgs A)
                 if (PEPS) s_e[q] = e2;
             }
             __syncthreads();
-            for (int c0 = 0; c0 < kTile; c0 += kChunk) {
-                float ca[R][3];
-#pragma unroll
-                for (int k = 0; k < R; ++k) ca[k][0] = ca[k][1] = ca[k][2] = 0.0f;
-#pragma unroll 4
-                for (int jj = c0; jj < c0 + kChunk; ++jj) {
-                    const float4 p = s_p[jj];
-                    const float e2 = PEPS ? s_e[jj] : f.eps2u;
-#pragma unroll
-                    for (int k = 0; k < R; ++k) {
-                        const float dx = rx[k] - p.x, dy = ry[k] - p.y, dz = rz[k] - p.z;
-                        const float dxx = dx * dx, dyy = dy * dy;
-                        const float r2 = fmaf(dz, dz, dxx + dyy) + e2;
-                        const float inv = rsqrt_mufu(r2);
-                        const float i2 = inv * inv;
-                        const float m3 = p.w * inv * i2, m5 = m3 * i2;
-                        ca[k][0] += fmaf(-3.0f * (dxx + dyy), m5, 2.0f * m3);
-                        ca[k][1] = fmaf(dyy - dxx, m5, ca[k][1]);
-                        ca[k][2] = fmaf(dx * dy, m5, ca[k][2]);
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < R; ++k)
-#pragma unroll
-                    for (int o2 = 0; o2 < 3; ++o2) two_sum_into(hi[k][o2], lo[k][o2], ca[k][o2]);
-            }
+            if (flat) hess_tile<R, PEPS, true>(s_p, s_e, f.eps2u, rx, ry, rz, hi, lo);
+            else hess_tile<R, PEPS, false>(s_p, s_e, f.eps2u, rx, ry, rz, hi, lo);
         }
     }
     float2 *out = (float2 *)A.out;
@@ -147,7 +168,10 @@ __global__ void __launch_bounds__(NT) k_hess(ForceArgs A)
         const int64_t i = base + (int64_t)k * NT + tid;
         if (i < A.n)
 #pragma unroll
-            for (int o2 = 0; o2 < 3; ++o2) out[((int64_t)split * 3 + o2) * A.n + i] = make_float2(hi[k][o2], lo[k][o2]);
+            for (int o2 = 0; o2 < 3; ++o2) {
+                const float c = o2 == 0 ? 2.0f : 1.0f;  // A was summed halved
+                out[((int64_t)split * 3 + o2) * A.n + i] = make_float2(c * hi[k][o2], c * lo[k][o2]);
+            }
     }
 }
 
