@@ -2004,6 +2004,7 @@ extern "C" int rt3d_load_grid(rt3d_ctx *ctx, int field_id, int64_t n, const doub
     fs.gd.n = g->n;
     fs.gd.n_int = g->n_int;
     fs.gd.h = g->h;
+    fs.gd.inv_h = 1.0 / g->h;
     for (int d = 0; d < 3; ++d) fs.gd.lo[d] = g->lo[d];
     int rc = grid_build(fs.gd, n, pos, mass, soft, g->mean_subtract ? 1 : 0, ctx->opt.precision == RT3D_FP64,
                         ctx->stream, ctx->err);
@@ -2059,6 +2060,7 @@ extern "C" int rt3d_load_grid_box(rt3d_ctx *ctx, int field_id, int64_t n, const 
     G.L = L;
     G.W = L / cubes;
     G.h = G.W / (g->n - 1);
+    G.inv_h = 1.0 / G.h;
     G.margin = 1.0;
     int rc = grid_build_box(G, n, pos, mass, soft, vol->rot, vol->shift, g->mean_subtract ? 1 : 0,
                             ctx->opt.precision == RT3D_FP64, ctx->stream, ctx->err);

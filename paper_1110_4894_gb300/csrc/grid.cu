@@ -301,7 +301,7 @@ __device__ __forceinline__ void grid_eval64_at(const GridDev &g, const double r[
     bool inside = true;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        u[d] = (r[d] - lo[d]) / g.h;
+        u[d] = grid_coord(r[d] - lo[d], g.h, g.inv_h);
         inside = inside && (u[d] >= -g.margin && u[d] <= (double)(n - 1) + g.margin);
         int sd = inside ? (int)floor(u[d]) - NI + 1 : 0;
         sd = sd > n - W ? n - W : sd;

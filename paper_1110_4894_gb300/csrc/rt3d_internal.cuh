@@ -372,7 +372,7 @@ constexpr int kGridRec = 8;
 struct GridDev {
     int n = 0, n_int = 0;
     double lo[3] = {0.0, 0.0, 0.0};
-    double h = 0.0;
+    double h = 0.0, inv_h = 0.0;  // node spacing and its inverse
     // one of the two: [i1][i2][i3][kGridRec], i3 fastest, in FP64 (FP64
     // contexts) or rounded to FP32 (mixed contexts)
     double *tab = nullptr;
