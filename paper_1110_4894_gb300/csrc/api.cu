@@ -1088,8 +1088,14 @@ static int trace_advance(rt3d_ctx *ctx, int n, cudaStream_t st)
     const int nr = T.rs.nr;
     Scratch &s = ctx->scr;
     const int stop = std::min(T.total, T.next + n);
-    if (fs.is_grid && !T.timed && T.next < stop) {  // all the stages in one launch (timed traces: kernel by kernel)
-        CK(launch_grid_trace(T.tp, fs.gd, T.rs, T.fp64, T.next, stop, s.dlam, s.misc, s.counters, st));
+    // fields that each ray evaluates for itself: all the stages in one launch
+    // (timed traces: kernel by kernel)
+    const bool few = T.fp64 && !fs.is_grid && !fs.df.replicated && fs.n <= kFewParticles;
+    if ((fs.is_grid || few) && !T.timed && T.next < stop) {
+        if (few)
+            CK(launch_few_trace(T.tp, fs.df, T.rs, T.next, stop, s.dlam, s.misc, s.counters, st));
+        else
+            CK(launch_grid_trace(T.tp, fs.gd, T.rs, T.fp64, T.next, stop, s.dlam, s.misc, s.counters, st));
         T.next = stop;
         T.launches += 1;
         T.flaunch += 1;

@@ -1246,20 +1246,6 @@ __global__ void __launch_bounds__(NT) k_force_bundle(ForceArgs A)
                                                    (float2 *)A.out, s_p, s_e);
 }
 
-// 1 / sqrt(x) of a positive FP64 number: the hardware's approximation y
-// (rsqrt.approx.ftz.f64, relative error 2^-20 or better, its low word zero, so
-// y^2 is exact), corrected by the binomial series (1 - e)^(-1/2) = 1 + e / 2 + 3
-// e^2 / 8 + ... for e = 1 - x y^2; the term left out is below 2^-61.  Five FP64
-// operations, no branch.  x = 0 gives infinity, as rsqrt does.
-__device__ __forceinline__ double rsqrt_series(double x)
-{
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y * y, 1.0), t = e * fma(e, 0.375, 0.5);
-    const double r = fma(y, t, y);
-    return __double2hiint(y) == 0x7ff00000 ? y : r;  // x = 0 (an integer compare)
-}
-
 // FP64 twin (the all-FP64 path): same staging, FP64 arithmetic, plain sums.
 // Bound by the FP64 pipe (2 lanes per SM): 18 operations per interaction.  The
 // particle loop ends at the last particle staged (rounded up to the unroll of
@@ -1331,14 +1317,7 @@ __global__ void __launch_bounds__(NT) k_force_fp64(ForceArgs A)
                     const double e2 = PEPS ? s_e[jj] : f.eps2u64;
 #pragma unroll
                     for (int k = 0; k < R; ++k) {
-                        const double dx = p.x - rx[k], dy = p.y - ry[k], dz = p.z - rz[k];
-                        const double inv = rsqrt_series(fma(dx, dx, fma(dy, dy, fma(dz, dz, e2))));
-                        const double mi = p.w * inv;
-                        const double mi3 = mi * (inv * inv);
-                        acc[k][0] += mi;
-                        acc[k][1] = fma(dx, mi3, acc[k][1]);
-                        acc[k][2] = fma(dy, mi3, acc[k][2]);
-                        acc[k][3] = fma(dz, mi3, acc[k][3]);
+                        pair_fp64(p.x - rx[k], p.y - ry[k], p.z - rz[k], p.w, e2, acc[k]);
                     }
                 }
             }

@@ -428,90 +428,26 @@ cudaError_t launch_grid_eval(const GridDev &g, const double *px, const double *p
 // ---------------------------------------------------------------------------
 // traces on a grid
 // ---------------------------------------------------------------------------
-// RK4 stages [g0, g1) of every ray in one launch.  On a grid nothing couples
-// the rays but the cube of their bundle's central ray, so a warp takes whole
-// bundles (6 of 5 rays, 3 of 9), keeps their states in registers and runs
-// through all the stages; the central ray's x3 comes by shuffle.  Stage by
-// stage, a trace was an evaluation and an update kernel per stage with the
-// state, the field and their launches between them: 11.5 + 5.9 us for 20,480
-// rays and a 128^3 grid; grid and trace of 500 steps together 75.6 -> 36.4 ms
-// (the grid was 20 ms of both).  What is left is each stage's
-// FP64 (about 150 operations per ray on two lanes per SM) behind the latency of
-// its node gather.  A bundle whose rays are all across stops: results are
-// taken at the crossing, and the stages after it only served other bundles.
-// One warp per block spreads a few hundred warps evenly over the SMs.
-constexpr int kGridTraceNT = 32;
-
+// trace_rays with the grid's interpolation.  Stage by stage, a trace was an
+// evaluation and an update kernel per stage with the state, the field and their
+// launches between them: 11.5 + 5.9 us for 20,480 rays and a 128^3 grid; grid
+// and trace of 500 steps together 75.6 -> 36.4 ms (the grid was 20 ms of both).
+// What is left is each stage's FP64 behind the latency of its node gather.
 template <int NI, bool FP64>
-__global__ void __launch_bounds__(kGridTraceNT) k_grid_trace(TraceParams tp, GridDev g, RayState rs, int g0, int g1,
+__global__ void __launch_bounds__(kTraceRaysNT) k_grid_trace(TraceParams tp, GridDev g, RayState rs, int g0, int g1,
                                                             const double *__restrict__ dlam,
                                                             const double *__restrict__ misc, unsigned long long *cnt)
 {
-    const int lane = threadIdx.x & 31, per_warp = 32 / rs.nr;
-    const int64_t b = (int64_t)blockIdx.x * per_warp + lane / rs.nr;
-    const bool valid = lane < per_warp * rs.nr && b < rs.n_b;
-    const int64_t i = valid ? b * rs.nr + lane % rs.nr : 0, st = rs.stride;
-    const int src = valid ? lane - lane % rs.nr : lane;  // the central ray's lane
-    double y[8], ys[8], ks[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        y[q] = rs.y[q * st + i];
-        ys[q] = rs.ys[q * st + i];
-        ks[q] = rs.ks[q * st + i];
-    }
-    bool done = !valid || rs.done[i] != 0;
-    const double chi_s = misc[0];
-    unsigned active = 0;
-    for (int s = g0; s < g1; ++s) {
-        const int step = s >> 2, stage = s & 3;
-        if ((stage == 0 || s == g0) && !__any_sync(0xffffffffu, !done)) break;
-        double F[4];
-        const double x3 = __shfl_sync(0xffffffffu, ys[3], src);
+    trace_rays(tp, rs, g0, g1, dlam, misc, cnt, [&](const double r[3], double x3, double F[4]) {
         if constexpr (FP64) {
-            grid_eval64_at<NI>(g, ys + 1, x3, F);
+            grid_eval64_at<NI>(g, r, x3, F);
         } else {
             float f[4];
-            grid_eval32_at<NI>(g, ys + 1, x3, f);
+            grid_eval32_at<NI>(g, r, x3, f);
 #pragma unroll
             for (int q = 0; q < 4; ++q) F[q] = (double)f[q];
         }
-        const double dl = dlam[step < tp.n_steps ? step : tp.n_steps - 1];
-        double k[8];
-        ray_slope(tp, ys, F, s == 0, y, k);
-        active += done ? 0u : 1u;
-        if (stage < 3) {
-            const double c = stage == 2 ? dl : 0.5 * dl;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                ks[q] = stage == 0 ? k[q] : ks[q] + 2.0 * k[q];
-                ys[q] = y[q] + c * k[q];
-            }
-        } else {
-            double nx[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) nx[q] = y[q] + dl * (1.0 / 6.0) * (ks[q] + k[q]);
-            if (!done && nx[3] >= chi_s) {
-                const double f = (chi_s - y[3]) / (nx[3] - y[3]);
-#pragma unroll
-                for (int q = 0; q < 8; ++q) rs.fin[q * st + i] = y[q] + f * (nx[q] - y[q]);
-                rs.done[i] = 1;
-                rs.steps[i] = step + 1;
-                done = true;
-            }
-#pragma unroll
-            for (int q = 0; q < 8; ++q) y[q] = ys[q] = nx[q];
-        }
-    }
-    if (valid) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            rs.y[q * st + i] = y[q];
-            rs.ys[q * st + i] = ys[q];
-            rs.ks[q * st + i] = ks[q];
-        }
-    }
-    const unsigned sum = __reduce_add_sync(0xffffffffu, valid ? active : 0u);
-    if (lane == 0 && sum) atomicAdd(&cnt[2], (unsigned long long)sum);
+    });
 }
 
 template <bool FP64>
@@ -521,10 +457,10 @@ static cudaError_t go_grid_trace(const TraceParams &tp, const GridDev &g, const 
     const int per_warp = 32 / rs.nr;
     const unsigned grid = (unsigned)((rs.n_b + per_warp - 1) / per_warp);
     switch (g.n_int) {
-    case 1: k_grid_trace<1, FP64><<<grid, kGridTraceNT, 0, st>>>(tp, g, rs, g0, g1, dlam, misc, cnt); break;
-    case 2: k_grid_trace<2, FP64><<<grid, kGridTraceNT, 0, st>>>(tp, g, rs, g0, g1, dlam, misc, cnt); break;
-    case 3: k_grid_trace<3, FP64><<<grid, kGridTraceNT, 0, st>>>(tp, g, rs, g0, g1, dlam, misc, cnt); break;
-    case 4: k_grid_trace<4, FP64><<<grid, kGridTraceNT, 0, st>>>(tp, g, rs, g0, g1, dlam, misc, cnt); break;
+    case 1: k_grid_trace<1, FP64><<<grid, kTraceRaysNT, 0, st>>>(tp, g, rs, g0, g1, dlam, misc, cnt); break;
+    case 2: k_grid_trace<2, FP64><<<grid, kTraceRaysNT, 0, st>>>(tp, g, rs, g0, g1, dlam, misc, cnt); break;
+    case 3: k_grid_trace<3, FP64><<<grid, kTraceRaysNT, 0, st>>>(tp, g, rs, g0, g1, dlam, misc, cnt); break;
+    case 4: k_grid_trace<4, FP64><<<grid, kTraceRaysNT, 0, st>>>(tp, g, rs, g0, g1, dlam, misc, cnt); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -257,6 +257,31 @@ __device__ __forceinline__ int replica_of(const DevField &f, double x3)
     return (int)q;
 }
 
+// 1 / sqrt(x) of a positive FP64 number: the hardware's approximation y
+// (rsqrt.approx.ftz.f64, relative error 2^-20 or better, its low word zero, so
+// y^2 is exact), corrected by the binomial series (1 - e)^(-1/2) = 1 + e / 2 + 3
+// e^2 / 8 + ... for e = 1 - x y^2; the term left out is below 2^-61.  Five FP64
+// operations, no branch.  x = 0 gives infinity, as rsqrt does.
+__device__ __forceinline__ double rsqrt_series(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y * y, 1.0), t = e * fma(e, 0.375, 0.5);
+    const double r = fma(y, t, y);
+    return __double2hiint(y) == 0x7ff00000 ? y : r;  // x = 0 (an integer compare)
+}
+
+// one particle of mass m at offset d: adds m / r and m d / r^3, r^2 = |d|^2 + e2
+__device__ __forceinline__ void pair_fp64(double dx, double dy, double dz, double m, double e2, double acc[4])
+{
+    const double inv = rsqrt_series(fma(dx, dx, fma(dy, dy, fma(dz, dz, e2))));
+    const double mi = m * inv, mi3 = mi * (inv * inv);
+    acc[0] += mi;
+    acc[1] = fma(dx, mi3, acc[1]);
+    acc[2] = fma(dy, mi3, acc[2]);
+    acc[3] = fma(dz, mi3, acc[3]);
+}
+
 // ---------------------------------------------------------------------------
 // ray state (SoA, FP64): index [component * n_rays + ray]
 // ---------------------------------------------------------------------------
@@ -347,6 +372,11 @@ inline double partial_mass_factor(const DevField &f, const ForceShape &sh)
 {
     return sh.umass ? f.m_uniform : 1.0;
 }
+// RK4 stages [g0, g1) of an FP64 trace through an isolated field of few particles
+constexpr int kFewParticles = 64;
+cudaError_t launch_few_trace(const TraceParams &tp, const DevField &f, const RayState &rs, int g0, int g1,
+                             const double *d_dlam, const double *d_misc, unsigned long long *d_counters,
+                             cudaStream_t st);
 cudaError_t launch_reduce(const TraceParams &tp, const double *d_theta, RayState rs, const double *d_misc,
                           double *d_bout, double *d_rout, cudaStream_t st);
 // words of d_scal: five counters, a ticket, three doubles per block

@@ -444,6 +444,80 @@ __device__ __forceinline__ bool stage_ray(const TraceParams &tp, const DevField 
     return !done;
 }
 
+// RK4 stages [g0, g1) of every ray, for a field that each ray evaluates for
+// itself: eval(r, x3, F) gives phi and grad phi at r, x3 the central ray's.
+// Nothing but that x3 then couples the rays, so a warp takes whole bundles (6 of
+// 5 rays, 3 of 9), keeps their states in registers and runs through all the
+// stages in one launch; x3 comes by shuffle.  The bound is FP64: about 150
+// operations per ray and stage on two lanes per SM, in a chain of some sixty.
+// A bundle whose rays are all across stops: results are taken at the crossing,
+// and the stages after it only served other bundles.  Blocks are one warp, which
+// spreads a few hundred warps evenly over the SMs.
+constexpr int kTraceRaysNT = 32;
+
+template <class Eval>
+__device__ __forceinline__ void trace_rays(const TraceParams &tp, const RayState &rs, int g0, int g1,
+                                           const double *__restrict__ dlam, const double *__restrict__ misc,
+                                           unsigned long long *cnt, const Eval &eval)
+{
+    const int lane = threadIdx.x & 31, per_warp = 32 / rs.nr;
+    const int64_t b = (int64_t)blockIdx.x * per_warp + lane / rs.nr;
+    const bool valid = lane < per_warp * rs.nr && b < rs.n_b;
+    const int64_t i = valid ? b * rs.nr + lane % rs.nr : 0, st = rs.stride;
+    const int src = valid ? lane - lane % rs.nr : lane;  // the central ray's lane
+    double y[8], ys[8], ks[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        y[q] = rs.y[q * st + i];
+        ys[q] = rs.ys[q * st + i];
+        ks[q] = rs.ks[q * st + i];
+    }
+    bool done = !valid || rs.done[i] != 0;
+    const double chi_s = misc[0];
+    unsigned active = 0;
+    for (int s = g0; s < g1; ++s) {
+        const int step = s >> 2, stage = s & 3;
+        if ((stage == 0 || s == g0) && !__any_sync(0xffffffffu, !done)) break;
+        const double dl = dlam[step < tp.n_steps ? step : tp.n_steps - 1];
+        double F[4], k[8];
+        eval(ys + 1, __shfl_sync(0xffffffffu, ys[3], src), F);
+        ray_slope(tp, ys, F, s == 0, y, k);
+        active += done ? 0u : 1u;
+        if (stage < 3) {
+            const double c = stage == 2 ? dl : 0.5 * dl;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                ks[q] = stage == 0 ? k[q] : ks[q] + 2.0 * k[q];
+                ys[q] = y[q] + c * k[q];
+            }
+        } else {
+            double nx[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) nx[q] = y[q] + dl * (1.0 / 6.0) * (ks[q] + k[q]);
+            if (!done && nx[3] >= chi_s) {
+                const double f = (chi_s - y[3]) / (nx[3] - y[3]);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) rs.fin[q * st + i] = y[q] + f * (nx[q] - y[q]);
+                rs.done[i] = 1;
+                rs.steps[i] = step + 1;
+                done = true;
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) y[q] = ys[q] = nx[q];
+        }
+    }
+    if (valid) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            rs.y[q * st + i] = y[q];
+            rs.ys[q * st + i] = ys[q];
+            rs.ks[q * st + i] = ks[q];
+        }
+    }
+    const unsigned sum = __reduce_add_sync(0xffffffffu, valid ? active : 0u);
+    if (lane == 0 && sum) atomicAdd(&cnt[2], (unsigned long long)sum);
+}
+
 // One bundle's lens-map Jacobian from its rays' states at x3 = chi_s; writes
 // (mu, kappa, gamma1, gamma2, omega, flags) to o[0..5] and, when rout is
 // given, each ray's final state to rout[(b * nr + k) * 8 + q].
