@@ -72,7 +72,7 @@ typedef struct {
     int threads_per_block; /* force-kernel block size (64..512); 0 = tuned */
     int splits;            /* particle splits per ray block; 0 = tuned */
     int autotune;          /* 1: time candidate launch shapes once per size bucket */
-    double watchdog_s;     /* limit for the persistent kernel's grid-barrier waits; 0 = 120 s */
+    double watchdog_s;     /* limit for the persistent kernel's waits; 0 = 120 s */
     int time_kernels;      /* 1: bracket every pair-sum launch with CUDA events (stats.force_ms) */
     int variant;           /* pair-sum kernel: 0 = automatic (bundle-centric FP32x2 for traces:
                               5 for rings of 4 and 8, 3 otherwise; with autotune, the fastest of
@@ -417,7 +417,7 @@ int rt3d_histogram_device(rt3d_ctx *ctx, void *stream, int64_t n, const double *
                           const rt3d_hist_opts *o, uint64_t *d_counts, uint64_t *d_wfix, double *d_scalars);
 
 /* Watchdog self-test (the paper has no counterpart): one GPU thread runs the
- * bounded wait of the persistent kernel's grid barrier on a device word that
+ * bounded wait of the persistent kernel's idle blocks on a device word that
  * nothing changes.  The wait must give up after limit_s (0 < limit_s <= 10)
  * and report it, leaving the context usable: the call then returns
  * RT3D_ETIMEOUT, which is the passing outcome; RT3D_ECUDA if the wait ended

@@ -238,6 +238,8 @@ struct rt3d_ctx {
         size_t cones_n = 0;
         int4 *items = nullptr;
         size_t items_n = 0;
+        int *order = nullptr;
+        size_t order_n = 0;
         int *rb2cone = nullptr;
         size_t rb_n = 0;
         double *state = nullptr;
@@ -252,7 +254,7 @@ struct rt3d_ctx {
         size_t partials_n = 0;
         unsigned long long *cnt = nullptr;
         size_t cnt_n = 0;
-        unsigned *bar = nullptr;  // [0] count, [1] generation, [2] error word, [4], [5] work queues
+        unsigned *bar = nullptr;  // [0] cones done, [1] events, [2] error word
         double *bout = nullptr;
         size_t bout_n = 0;
         double *rout = nullptr;
@@ -394,6 +396,7 @@ extern "C" int rt3d_destroy(rt3d_ctx *ctx)
         if (B.exec) cudaGraphExecDestroy(B.exec);
         cudaFree(B.cones);
         cudaFree(B.items);
+        cudaFree(B.order);
         cudaFree(B.rb2cone);
         cudaFree(B.state);
         cudaFree(B.ints);
@@ -1407,14 +1410,15 @@ struct BatchPlan {
     std::vector<int64_t> ray_base, b_base, dlam_off, part_off, per_split;
     std::vector<int> S;
     std::vector<int4> items;
-    std::vector<int64_t> cost;  // rays x particles of each item (planning order)
+    std::vector<int64_t> item_base, cost;  // per cone: its first item; its pair interactions per stage
+    std::vector<int> order;                // the cones, most expensive first
     std::vector<int> rb2cone;
     size_t cone_bytes(int n) const { return sizeof(BatchCone) * (size_t)n; }
 };
 
 // Layout of a batch: each cone's rays padded to whole ray blocks of RB, its
 // particles split into whole tiles of about per_item particles, one work item
-// per (cone, ray block, split).
+// per (cone, ray block, split), cone by cone.
 static int plan_batch(const FieldSlot *fields, int n_cones, const rt3d_cone *cones, int nr, int RB, int NT,
                       int64_t per_item, int max_extra, BatchPlan &p)
 {
@@ -1422,7 +1426,10 @@ static int plan_batch(const FieldSlot *fields, int n_cones, const rt3d_cone *con
     for (int c = 0; c < n_cones; ++c) {
         const int64_t nb = cones[c].n_bundles, n_rays = nb * nr, N = fields[cones[c].field_id].n;
         const int64_t nrb = (n_rays + RB - 1) / RB;
+        p.item_base.push_back((int64_t)p.items.size());
+        p.cost.push_back(n_rays * std::max<int64_t>(N, 1));
         if (fields[cones[c].field_id].is_grid) {
+            p.cost.back() = 25 * n_rays;  // about 500 FP32 operations and 1 KB of node reads per ray
             // a grid cone: one evaluation item per ray block, one split
             p.ray_base.push_back(p.T);
             p.b_base.push_back(p.n_b_total);
@@ -1432,8 +1439,6 @@ static int plan_batch(const FieldSlot *fields, int n_cones, const rt3d_cone *con
             p.S.push_back(1);
             for (int64_t rb = 0; rb < nrb; ++rb) {
                 p.items.push_back(make_int4(c, (int)rb, 0, 1));
-                // about 500 FP32 operations and 1 KB of node reads per ray
-                p.cost.push_back(25 * std::min<int64_t>(RB, n_rays - rb * RB));
                 p.rb2cone.push_back(c);
             }
             p.T += nrb * RB;
@@ -1455,46 +1460,32 @@ static int plan_batch(const FieldSlot *fields, int n_cones, const rt3d_cone *con
         p.part_off.push_back(p.partials_total);
         p.per_split.push_back(tps * kTile);
         p.S.push_back((int)S);
+        const FieldSlot &fs = fields[cones[c].field_id];
+        if (fs.df.replicated && fs.df.mean_subtract) {
+            // prism records: one item per block of NT bundles, first in the phase
+            const int64_t nbb = (nb + NT - 1) / NT;
+            for (int64_t q = 0; q < nbb; ++q) p.items.push_back(make_int4(c, (int)q, -1, 0));
+        }
         for (int64_t rb = 0; rb < nrb; ++rb) {
             for (int64_t s = 0; s < S; ++s) p.items.push_back(make_int4(c, (int)rb, (int)s, 0));
             p.rb2cone.push_back(c);
         }
         p.T += nrb * RB;
-        const FieldSlot &fs = fields[cones[c].field_id];
-        if (fs.df.replicated && fs.df.mean_subtract) {
-            // prism records: one item per block of NT bundles, costed as the
-            // FP64 closed form (about 24 000 pair interactions per bundle)
-            const int64_t nbb = (nb + NT - 1) / NT;
-            for (int64_t q = 0; q < nbb; ++q) {
-                p.items.push_back(make_int4(c, (int)q, -1, 0));
-                p.cost.push_back(24000 * std::min<int64_t>(NT, nb - q * NT));
-            }
-        }
-        for (int64_t rb = 0; rb < nrb; ++rb) {
-            const int64_t rays = std::min<int64_t>(RB, n_rays - rb * RB);
-            for (int64_t s = 0; s < S; ++s) {
-                const int64_t parts = std::min<int64_t>(tps * kTile, N - s * tps * kTile);
-                p.cost.push_back(rays * std::max<int64_t>(parts, 1));
-            }
-        }
         p.n_b_total += nb;
         p.dlam_total += cones[c].n_steps;
         p.partials_total += S * 4 * n_rays;
         p.max_steps = std::max(p.max_steps, cones[c].n_steps);
         p.g_end = std::max(p.g_end, 4 * (cones[c].n_steps + max_extra));
     }
-    // the work queue hands out items in this order: largest first
-    std::vector<size_t> order(p.items.size());
-    for (size_t i = 0; i < order.size(); ++i) order[i] = i;
-    std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) { return p.cost[a] > p.cost[b]; });
-    std::vector<int4> sorted(p.items.size());
-    for (size_t i = 0; i < order.size(); ++i) sorted[i] = p.items[order[i]];
-    p.items.swap(sorted);
+    p.item_base.push_back((int64_t)p.items.size());
+    p.order.resize((size_t)n_cones);
+    for (int c = 0; c < n_cones; ++c) p.order[(size_t)c] = c;
+    std::stable_sort(p.order.begin(), p.order.end(), [&](int a, int b) { return p.cost[a] > p.cost[b]; });
     return RT3D_OK;
 }
 
 static void fill_cone_table(const FieldSlot *fields, const Cosmo &cosmo, int christoffel, int n_cones,
-                            const rt3d_cone *cones, const rt3d_bundle_opts *b, const BatchPlan &p, double *state,
+                            const rt3d_cone *cones, const rt3d_bundle_opts *b, const BatchPlan &p, int NT, double *state,
                             int *ints, double *theta, double *dlam, float2 *partials, unsigned long long *cnt,
                             double *rout, double *prism, std::vector<unsigned char> &table)
 {
@@ -1545,6 +1536,9 @@ static void fill_cone_table(const FieldSlot *fields, const Cosmo &cosmo, int chr
         C.total_steps = cones[c].n_steps + b->max_extra;
         C.grid = fields[cones[c].field_id].is_grid ? 1 : 0;
         C.g = fields[cones[c].field_id].gd;
+        C.item_base = p.item_base[c];
+        C.n_force = (int)(p.item_base[c + 1] - p.item_base[c]);
+        C.n_stage = (int)((rs.n_rays + NT - 1) / NT);
     }
 }
 
@@ -1585,6 +1579,7 @@ static int batch_run(rt3d_ctx *ctx, int n_cones, const rt3d_cone *cones, const r
     const int64_t T = plan.T;
     CK(grow(*(char **)&BS.cones, BS.cones_n, plan.cone_bytes(n_cones)));
     CK(grow(BS.items, BS.items_n, plan.items.size()));
+    CK(grow(BS.order, BS.order_n, plan.order.size()));
     CK(grow(BS.rb2cone, BS.rb_n, plan.rb2cone.size()));
     CK(grow(BS.state, BS.state_n, (size_t)(32 * T)));
     CK(grow(BS.ints, BS.ints_n, (size_t)(2 * T + 2 * plan.n_b_total)));
@@ -1598,7 +1593,7 @@ static int batch_run(rt3d_ctx *ctx, int n_cones, const rt3d_cone *cones, const r
     if (want_rays) CK(grow(BS.rout, BS.rout_n, (size_t)(8 * nr * plan.n_b_total)));
     std::vector<unsigned char> table;
     CK(grow(BS.prism, BS.prism_n, (size_t)(kPrismRec * plan.n_b_total)));
-    fill_cone_table(ctx->fields.data(), ctx->cosmo, ctx->opt.christoffel, n_cones, cones, b, plan, BS.state, BS.ints,
+    fill_cone_table(ctx->fields.data(), ctx->cosmo, ctx->opt.christoffel, n_cones, cones, b, plan, NT, BS.state, BS.ints,
                     BS.theta, BS.dlam, BS.partials, BS.cnt, want_rays ? BS.rout : nullptr, BS.prism, table);
     cudaStream_t st = ctx->stream;
     for (int c = 0; c < n_cones; ++c)
@@ -1606,18 +1601,20 @@ static int batch_run(rt3d_ctx *ctx, int n_cones, const rt3d_cone *cones, const r
                            cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(BS.cones, table.data(), table.size(), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(BS.items, plan.items.data(), plan.items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(BS.order, plan.order.data(), plan.order.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(BS.rb2cone, plan.rb2cone.data(), plan.rb2cone.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     CK(cudaMemsetAsync(BS.bar, 0, 8 * sizeof(unsigned), st));
     int grid = 0;
     CK(batch_resident_blocks(NT, MODE, &grid));
     if (grid < 1) return fail(ctx, RT3D_ECUDA, "persistent kernel cannot be resident");
-    BatchArgs A = make_batch_args(BS.cones, n_cones, BS.items, (int64_t)plan.items.size(), BS.rb2cone, T, RB,
+    BatchArgs A = make_batch_args(BS.cones, n_cones, BS.items, (int64_t)plan.items.size(), BS.order, BS.rb2cone, T, RB,
                                   g_limit > 0 ? g_limit : plan.g_end, BS.bar, (int *)(BS.bar + 2),
                                   ctx->opt.watchdog_s > 0 ? ctx->opt.watchdog_s : 120.0, BS.bout);
     // the graph is keyed by everything its launches capture
     std::vector<long long> key = {n_cones, T, (long long)plan.items.size(), A.g_end, NT, MODE, per_item, grid,
                                   plan.max_steps, plan.n_b_total, (long long)(intptr_t)BS.cones,
-                                  (long long)(intptr_t)BS.items, (long long)(intptr_t)BS.bout,
+                                  (long long)(intptr_t)BS.items, (long long)(intptr_t)BS.order,
+                                  (long long)(intptr_t)BS.rb2cone, (long long)(intptr_t)BS.bout,
                                   (long long)(intptr_t)BS.prism};
     CK(cudaEventRecord(ctx->ev0, st));
     bool use_graph = g_limit == 0;
@@ -1655,7 +1652,7 @@ static int batch_run(rt3d_ctx *ctx, int n_cones, const rt3d_cone *cones, const r
     if (ms_out) *ms_out = ms;
     unsigned err = 0;
     CK(cudaMemcpy(&err, BS.bar + 2, sizeof err, cudaMemcpyDeviceToHost));
-    if (err) return fail(ctx, RT3D_ETIMEOUT, "persistent kernel: a grid barrier wait exceeded the watchdog");
+    if (err) return fail(ctx, RT3D_ETIMEOUT, "persistent kernel: a wait exceeded the watchdog");
     ctx->stats.device_ms = ms;
     ctx->stats.launches = 4;
     ctx->stats.force_launches = 1;

@@ -21,7 +21,14 @@ struct BatchCone {
     int S, flags, total_steps, kind;
     int grid;              // 1: the field is a grid (g), read by grid items; S = 1
     GridDev g;
+    // the cone's place in its work: phase 2 g is the force items of stage g,
+    // phase 2 g + 1 its stage items (NT rays each)
+    int64_t item_base;     // its force items in the items array
+    int n_force, n_stage;  // items of the two kinds of phase
+    unsigned long long word;  // phase << 32 | next item (zero at the launch)
+    unsigned finished;        // items of the phase that are done
 };
+constexpr unsigned kBatchDone = 0xffffffffu;  // phase of a cone that is done
 
 struct BatchArgs {
     BatchCone *cones;
@@ -29,18 +36,19 @@ struct BatchArgs {
     const int4 *items;     // (cone, ray block, split, kind); split -1: the prism records of a
                            // block of NT bundles; kind 1: grid evaluation of a ray block
     int64_t n_items;
+    const int *order;      // the cones, most expensive first
     const int *rb2cone;    // cone of each padded ray block
     int64_t T;             // padded ray count
     int RB;                // rays per block
     int g_end;             // global stages to run
-    unsigned *bar;         // [0] barrier count, [1] generation, [2] error word, [4], [5] work queues
+    unsigned *bar;         // [0] cones that are done, [1] events, [2] error word
     int *err;              // watchdog / error word
     unsigned long long limit_ns;
     double *bout;
 };
 
-inline BatchArgs make_batch_args(void *cones, int n_cones, const int4 *items, int64_t n_items, const int *rb2cone,
-                                 int64_t T, int RB, int g_end, unsigned *bar, int *err, double watchdog_s,
+inline BatchArgs make_batch_args(void *cones, int n_cones, const int4 *items, int64_t n_items, const int *order,
+                                 const int *rb2cone, int64_t T, int RB, int g_end, unsigned *bar, int *err, double watchdog_s,
                                  double *bout)
 {
     BatchArgs A;
@@ -48,6 +56,7 @@ inline BatchArgs make_batch_args(void *cones, int n_cones, const int4 *items, in
     A.n_cones = n_cones;
     A.items = items;
     A.n_items = n_items;
+    A.order = order;
     A.rb2cone = rb2cone;
     A.T = T;
     A.RB = RB;
