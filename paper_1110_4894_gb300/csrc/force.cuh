@@ -1115,9 +1115,8 @@ __global__ void __launch_bounds__(NT, TPSM / NT) k_force_bundle2x(ForceArgs A)
 // two-bundle kernel, so the results are the same bits.  One tile per block
 // (blockIdx.y); a block holds NT / NR whole bundles.
 template <int NT, int NRING, bool REPL, bool PEPS, bool UMASS>
-__global__ void __launch_bounds__(NT) k_force_bundle1(ForceArgs A, int group)
+__global__ void __launch_bounds__(NT, 1) k_force_bundle1(ForceArgs A, int group)
 {
-    if (A.gate && *A.gate == 0ull) return;
     constexpr int NR = NRING + 1, BPB = NT / NR;
     __shared__ float4 s_p[kTile];
     __shared__ float s_e[PEPS ? kTile : 1];
@@ -1125,6 +1124,16 @@ __global__ void __launch_bounds__(NT) k_force_bundle1(ForceArgs A, int group)
     __shared__ int s_rmin, s_rmax;
     const DevField &f = A.f;
     const int tid = threadIdx.x, split = blockIdx.y;
+    let_next_start();
+    // the tile's particles are the field's: they are read ahead of the wait
+    const int64_t p0 = (int64_t)split * kTile;
+    const int cnt = (int)min((int64_t)kTile, f.n - p0);
+    int4 part[kTile / NT];
+#pragma unroll
+    for (int k = 0; k < kTile / NT; ++k)
+        if (k * NT + tid < cnt) part[k] = f.part[p0 + k * NT + tid];
+    wait_for_previous();
+    if (A.gate && *A.gate == 0ull) return;
     const int per_group = (group + BPB - 1) / BPB;
     const int64_t g0 = (int64_t)(blockIdx.x / per_group) * group;  // the group's first bundle
     const int first = (int)(blockIdx.x % per_group) * BPB;         // the block's first bundle in the group
@@ -1156,8 +1165,6 @@ __global__ void __launch_bounds__(NT) k_force_bundle1(ForceArgs A, int group)
     }
     float hx = 0.f, hy = 0.f, hz = 0.f, hs = 0.f, lx = 0.f, ly = 0.f, lz = 0.f, ls = 0.f, phi = 0.f;
     const float dlt = (float)f.delta;
-    const int64_t p0 = (int64_t)split * kTile;
-    const int cnt = (int)min((int64_t)kTile, f.n - p0);
     for (int j = rmin; j <= rmax; ++j) {
         if (!__syncthreads_or(myrep == j)) continue;  // no point of this block is in replica j
         double o[3];
@@ -1171,9 +1178,11 @@ __global__ void __launch_bounds__(NT) k_force_bundle1(ForceArgs A, int group)
             ny = -(float)(((A.py[ic] - o[1]) * f.inv_delta - (double)ay) * f.delta);
             nz = -(float)(((A.pz[ic] - o[2]) * f.inv_delta - (double)az) * f.delta);
         }
-#pragma unroll 4
-        for (int q = tid; q < cnt; q += NT) {
-            const int4 pr = f.part[p0 + q];
+#pragma unroll
+        for (int k = 0; k < kTile / NT; ++k) {
+            const int q = k * NT + tid;
+            if (q >= cnt) break;
+            const int4 pr = part[k];
             long long qq[3] = {pr.x, pr.y, pr.z};
             if (REPL) replica_q(f, j, pr.x, pr.y, pr.z, qq);
             s_p[q] = make_float4((float)(qq[0] - ax) * dlt, (float)(qq[1] - ay) * dlt, (float)(qq[2] - az) * dlt,
@@ -1256,6 +1265,8 @@ __global__ void __launch_bounds__(NT) k_force_bundle(ForceArgs A)
 template <int R, int NT, bool REPL, bool PEPS>
 __global__ void __launch_bounds__(NT) k_force_fp64(ForceArgs A)
 {
+    let_next_start();
+    wait_for_previous();
     if (A.gate && *A.gate == 0ull) return;
     __shared__ double4_16a s_p[kTile64];
     __shared__ double s_e[PEPS ? kTile64 : 1];

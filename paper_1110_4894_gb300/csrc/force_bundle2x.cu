@@ -74,11 +74,9 @@ static cudaError_t go_lanes(const ForceArgs &A, int group, int splits, cudaStrea
     // whole groups, then the blocks that the last group's bundles need
     const int64_t full = n_b / group, rest = n_b % group;
     const dim3 grid((unsigned)(full * ((group + BPB - 1) / BPB) + (rest + BPB - 1) / BPB), (unsigned)splits);
-    if (repl && peps) k_force_bundle1<NT, NRING, true, true, UMASS><<<grid, NT, 0, st>>>(A, group);
-    else if (repl) k_force_bundle1<NT, NRING, true, false, UMASS><<<grid, NT, 0, st>>>(A, group);
-    else if (peps) k_force_bundle1<NT, NRING, false, true, UMASS><<<grid, NT, 0, st>>>(A, group);
-    else k_force_bundle1<NT, NRING, false, false, UMASS><<<grid, NT, 0, st>>>(A, group);
-    return cudaGetLastError();
+    const auto kern = repl ? (peps ? k_force_bundle1<NT, NRING, true, true, UMASS> : k_force_bundle1<NT, NRING, true, false, UMASS>)
+                           : (peps ? k_force_bundle1<NT, NRING, false, true, UMASS> : k_force_bundle1<NT, NRING, false, false, UMASS>);
+    return launch_overlapped(kern, grid, NT, st, A, group);
 }
 
 // one ray per lane (one tile per split): one-warp blocks while a tile's rays fit

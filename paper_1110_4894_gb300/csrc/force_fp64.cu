@@ -7,11 +7,9 @@ template <int R, int NT>
 static cudaError_t go_fp64(const ForceArgs &A, dim3 grid, cudaStream_t st)
 {
     const bool repl = A.f.replicated != 0, peps = A.f.eps2_64 != nullptr;
-    if (repl && peps) k_force_fp64<R, NT, true, true><<<grid, NT, 0, st>>>(A);
-    else if (repl) k_force_fp64<R, NT, true, false><<<grid, NT, 0, st>>>(A);
-    else if (peps) k_force_fp64<R, NT, false, true><<<grid, NT, 0, st>>>(A);
-    else k_force_fp64<R, NT, false, false><<<grid, NT, 0, st>>>(A);
-    return cudaGetLastError();
+    const auto kern = repl ? (peps ? k_force_fp64<R, NT, true, true> : k_force_fp64<R, NT, true, false>)
+                           : (peps ? k_force_fp64<R, NT, false, true> : k_force_fp64<R, NT, false, false>);
+    return launch_overlapped(kern, grid, NT, st, A);
 }
 
 cudaError_t dispatch_fp64(const ForceArgs &A, const ForceShape &sh, cudaStream_t st)

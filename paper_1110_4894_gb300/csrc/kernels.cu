@@ -94,14 +94,18 @@ int device_sm_count()
     return sms;
 }
 
+// (The kernels below are launched overlapped: no pointer of theirs is declared
+// __restrict__, which would let its loads move ahead of the wait.)
 // the bundles' prism records of this stage (mean-subtracted boxes), read by
 // every ray of the bundle in k_stage: one warp per block, four bundles of eight
 // lanes, so that few bundles still use the FP64 lanes of many SMs
 constexpr int kPrismBundles = 32 / kCorners;
 __global__ void __launch_bounds__(32) k_prism(TraceParams tp, DevField f, RayState rs, int step, int stage,
-                                              const unsigned long long *cnt, double *__restrict__ prism)
+                                              const unsigned long long *cnt, double *prism)
 {
     __shared__ double s_q[kPrismBundles][10 * kCorners];
+    let_next_start();
+    wait_for_previous();
     if (step >= tp.n_steps && cnt[(step - 1) & 1] == 0ull) return;  // every ray is across
     const int k = threadIdx.x / kCorners;
     const int64_t b = (int64_t)blockIdx.x * kPrismBundles + k;
@@ -112,16 +116,18 @@ cudaError_t launch_prism(const TraceParams &tp, const DevField &f, RayState rs, 
                          const unsigned long long *d_counters, double *d_prism, cudaStream_t st)
 {
     const int64_t blocks = (rs.n_b + kPrismBundles - 1) / kPrismBundles;
-    k_prism<<<(unsigned)(blocks > 0 ? blocks : 1), 32, 0, st>>>(tp, f, rs, step, stage, d_counters, d_prism);
-    return cudaGetLastError();
+    return launch_overlapped(k_prism, dim3((unsigned)(blocks > 0 ? blocks : 1)), 32, st, tp, f, rs, step, stage,
+                             d_counters, d_prism);
 }
 
 __global__ void __launch_bounds__(kStageThreads) k_stage(TraceParams tp, DevField f, RayState rs, int S, int fp64,
-                                                        double mfac, const float2 *__restrict__ partials,
-                                                        const double *__restrict__ dlam,
-                                                        const double *__restrict__ misc, int step, int stage,
-                                                        unsigned long long *cnt, const double *__restrict__ prism)
+                                                        double mfac, const float2 *partials,
+                                                        const double *dlam,
+                                                        const double *misc, int step, int stage,
+                                                        unsigned long long *cnt, const double *prism)
 {
+    let_next_start();
+    wait_for_previous();
     if (stage == 0 && blockIdx.x == 0 && threadIdx.x == 0) cnt[step & 1] = 0ull;
     if (step >= tp.n_steps && cnt[(step - 1) & 1] == 0ull) return;  // every ray is across
     __shared__ double s_acc[kStageRays][4];
@@ -171,11 +177,13 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(TraceParams tp, DevFiel
 // splits (the grid path) or enough rays to fill the GPU, where the FP64
 // stage, not the reduction, needs the threads.
 __global__ void __launch_bounds__(256) k_stage_wide(TraceParams tp, DevField f, RayState rs, int S, int fp64,
-                                                   double mfac, const void *__restrict__ partials,
-                                                   const double *__restrict__ dlam,
-                                                   const double *__restrict__ misc, int step, int stage,
-                                                   unsigned long long *cnt, const double *__restrict__ prism)
+                                                   double mfac, const void *partials,
+                                                   const double *dlam,
+                                                   const double *misc, int step, int stage,
+                                                   unsigned long long *cnt, const double *prism)
 {
+    let_next_start();
+    wait_for_previous();
     if (stage == 0 && blockIdx.x == 0 && threadIdx.x == 0) cnt[step & 1] = 0ull;
     if (step >= tp.n_steps && cnt[(step - 1) & 1] == 0ull) return;  // every ray is across
     __shared__ unsigned s_active;
@@ -208,14 +216,13 @@ cudaError_t launch_stage(const TraceParams &tp, const DevField &f, RayState rs, 
         int nt = 256;
         while (nt > 32 && rs.n_rays < 2 * (int64_t)device_sm_count() * nt) nt /= 2;
         const int64_t blocks = (rs.n_rays + nt - 1) / nt;
-        k_stage_wide<<<(unsigned)blocks, nt, 0, st>>>(tp, f, rs, S, fp64 ? 1 : 0, mfac, d_partials, d_dlam, d_misc,
-                                                      step, stage, d_counters, d_prism);
+        return launch_overlapped(k_stage_wide, dim3((unsigned)blocks), nt, st, tp, f, rs, S, fp64 ? 1 : 0, mfac,
+                                 d_partials, d_dlam, d_misc, step, stage, d_counters, d_prism);
     } else {
         const int64_t blocks = (rs.n_rays + kStageRays - 1) / kStageRays;
-        k_stage<<<(unsigned)blocks, kStageThreads, 0, st>>>(tp, f, rs, S, fp64 ? 1 : 0, mfac, (const float2 *)d_partials,
-                                                            d_dlam, d_misc, step, stage, d_counters, d_prism);
+        return launch_overlapped(k_stage, dim3((unsigned)blocks), kStageThreads, st, tp, f, rs, S, fp64 ? 1 : 0, mfac,
+                                 (const float2 *)d_partials, d_dlam, d_misc, step, stage, d_counters, d_prism);
     }
-    return cudaGetLastError();
 }
 
 // trace_rays in FP64 through an isolated field of at most kFewParticles

@@ -46,3 +46,33 @@ def test_one_ray_lanes_give_the_same_bits(n_ring, bundles, n, varied, box):
         ctx.close()
     for k in res[0]:
         assert np.array_equal(res[0][k], res[1][k]), k
+
+
+@pytest.mark.parametrize("box", [False, True])
+def test_captured_trace_replays(box):
+    """the overlapped launches of a trace, captured into a CUDA graph and replayed, give the same bits"""
+    import torch
+
+    import paper_1110_4894_gb300 as P
+    pos, mass, soft, vol = case(700, False, box)
+    theta = torch.from_numpy(np.array([3e-4, -2e-4]) + 2e-4 * inputs.rng(7).normal(size=(5, 2))).cuda()
+    out = [torch.zeros((5, 6), dtype=torch.float64, device="cuda") for _ in range(2)]
+    ctx = P.Context(0)
+    ctx.set_cosmology(0.3, 0.7, 0.7)
+    ctx.load_particles(0, pos, mass, soft, **vol)
+
+    def trace(o):
+        ctx.trace_device(torch.cuda.current_stream().cuda_stream, 0, 0.5, 5, theta.data_ptr(), o.data_ptr(), n_ring=4,
+                         theta_r=5e-6, n_steps=12)
+
+    trace(out[0])  # sizes the context's scratch
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        trace(out[1])
+    for _ in range(3):
+        out[1].zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out[0], out[1])
+    ctx.close()
