@@ -142,15 +142,16 @@ __global__ void __launch_bounds__(NT) k_hess(ForceArgs A)
         flat = __syncthreads_and(flat) != 0;
         for (int64_t t0 = p0; t0 < p1; t0 += kTile) {
             __syncthreads();
+            const ReplicaMap rm = REPL ? replica_map(f, j) : ReplicaMap{};
             for (int q = tid; q < kTile; q += NT) {
                 const int64_t pi = t0 + q;
                 float4 v = make_float4(1e18f, 1e18f, 1e18f, 0.0f);
                 float e2 = 0.0f;
                 if (pi < p1) {
                     const int4 pr = f.part[pi];
-                    long long qq[3] = {pr.x, pr.y, pr.z};
-                    if (REPL) replica_q(f, j, pr.x, pr.y, pr.z, qq);
-                    v = make_float4((float)(qq[0] - ax) * dlt, (float)(qq[1] - ay) * dlt, (float)(qq[2] - az) * dlt,
+                    int qq[3] = {pr.x, pr.y, pr.z};
+                    if (REPL) replica_q(rm, pr.x, pr.y, pr.z, qq);
+                    v = make_float4(grid_offset(qq[0], ax) * dlt, grid_offset(qq[1], ay) * dlt, grid_offset(qq[2], az) * dlt,
                                     __int_as_float(pr.w));
                     if (PEPS) e2 = f.eps2[pi];
                 }

@@ -158,16 +158,17 @@ __global__ void __launch_bounds__(NT) k_force_mixed(ForceArgs A)
         }
         for (int64_t t0 = p0; t0 < p1; t0 += kTile) {
             __syncthreads();
+            const ReplicaMap rm = REPL ? replica_map(f, j) : ReplicaMap{};
             for (int q = tid; q < kTile; q += NT) {
                 const int64_t pi = t0 + q;
                 float4 v = make_float4(1e18f, 1e18f, 1e18f, 0.0f);
                 float e2 = 0.0f;
                 if (pi < p1) {
                     const int4 pr = f.part[pi];
-                    long long qq[3] = {pr.x, pr.y, pr.z};
-                    if (REPL) replica_q(f, j, pr.x, pr.y, pr.z, qq);
-                    v = make_float4((float)(qq[0] - ax) * dlt, (float)(qq[1] - ay) * dlt,
-                                    (float)(qq[2] - az) * dlt, __int_as_float(pr.w));
+                    int qq[3] = {pr.x, pr.y, pr.z};
+                    if (REPL) replica_q(rm, pr.x, pr.y, pr.z, qq);
+                    v = make_float4(grid_offset(qq[0], ax) * dlt, grid_offset(qq[1], ay) * dlt,
+                                    grid_offset(qq[2], az) * dlt, __int_as_float(pr.w));
                     if (PEPS) e2 = f.eps2[pi];
                 }
                 s_p[q] = v;
@@ -290,16 +291,17 @@ __device__ __forceinline__ void packed_block_sum(const DevField &f, const double
         }
         for (int64_t t0 = p0; t0 < p1; t0 += kTile) {
             __syncthreads();
+            const ReplicaMap rm = REPL ? replica_map(f, j) : ReplicaMap{};
             for (int q = tid; q < kTile; q += NT) {
                 const int64_t pi = t0 + q;
                 float x = 1e18f, y = 1e18f, z = 1e18f, m = 0.0f, e2 = 0.0f;
                 if (pi < p1) {
                     const int4 pr = f.part[pi];
-                    long long qq[3] = {pr.x, pr.y, pr.z};
-                    if (REPL) replica_q(f, j, pr.x, pr.y, pr.z, qq);
-                    x = (float)(qq[0] - ax) * dlt;
-                    y = (float)(qq[1] - ay) * dlt;
-                    z = (float)(qq[2] - az) * dlt;
+                    int qq[3] = {pr.x, pr.y, pr.z};
+                    if (REPL) replica_q(rm, pr.x, pr.y, pr.z, qq);
+                    x = grid_offset(qq[0], ax) * dlt;
+                    y = grid_offset(qq[1], ay) * dlt;
+                    z = grid_offset(qq[2], az) * dlt;
                     m = __int_as_float(pr.w);
                     if (PEPS) e2 = f.eps2[pi];
                 }
@@ -472,15 +474,16 @@ __device__ __forceinline__ void bundle_block_sum(const DevField &f, const double
         }
         for (int64_t t0 = p0; t0 < p1; t0 += kTile) {
             __syncthreads();
+            const ReplicaMap rm = REPL ? replica_map(f, j) : ReplicaMap{};
             for (int q = tid; q < kTile; q += NT) {
                 const int64_t pi = t0 + q;
                 float4 v = make_float4(1e18f, 1e18f, 1e18f, 0.0f);
                 float e2 = 0.0f;
                 if (pi < p1) {
                     const int4 pr = f.part[pi];
-                    long long qq[3] = {pr.x, pr.y, pr.z};
-                    if (REPL) replica_q(f, j, pr.x, pr.y, pr.z, qq);
-                    v = make_float4((float)(qq[0] - ax) * dlt, (float)(qq[1] - ay) * dlt, (float)(qq[2] - az) * dlt,
+                    int qq[3] = {pr.x, pr.y, pr.z};
+                    if (REPL) replica_q(rm, pr.x, pr.y, pr.z, qq);
+                    v = make_float4(grid_offset(qq[0], ax) * dlt, grid_offset(qq[1], ay) * dlt, grid_offset(qq[2], az) * dlt,
                                     __int_as_float(pr.w));
                     if (PEPS) e2 = f.eps2[pi];
                 }
@@ -651,16 +654,17 @@ __device__ __forceinline__ void bundle2_block_sum(const DevField &f, const doubl
                      NZ = make_float2(nc[0][2], nc[1][2]);
         for (int64_t t0 = p0; t0 < p1; t0 += kTile) {
             __syncthreads();
+            const ReplicaMap rm = REPL ? replica_map(f, j) : ReplicaMap{};
             for (int q = tid; q < kTile; q += NT) {
                 const int64_t pi = t0 + q;
                 float x = 1e18f, y = 1e18f, z = 1e18f, m = 0.0f, e2 = 0.0f;
                 if (pi < p1) {
                     const int4 pr = f.part[pi];
-                    long long qq[3] = {pr.x, pr.y, pr.z};
-                    if (REPL) replica_q(f, j, pr.x, pr.y, pr.z, qq);
-                    x = (float)(qq[0] - ax) * dlt;
-                    y = (float)(qq[1] - ay) * dlt;
-                    z = (float)(qq[2] - az) * dlt;
+                    int qq[3] = {pr.x, pr.y, pr.z};
+                    if (REPL) replica_q(rm, pr.x, pr.y, pr.z, qq);
+                    x = grid_offset(qq[0], ax) * dlt;
+                    y = grid_offset(qq[1], ay) * dlt;
+                    z = grid_offset(qq[2], az) * dlt;
                     m = __int_as_float(pr.w);
                     if (PEPS) e2 = f.eps2[pi];
                 }
@@ -867,16 +871,17 @@ __device__ __forceinline__ void bundle2x_block_sum(const DevField &f, const doub
                      NZ = make_float2(nc[0][2], nc[1][2]);
         for (int64_t t0 = p0; t0 < p1; t0 += kTile) {
             __syncthreads();
+            const ReplicaMap rm = REPL ? replica_map(f, j) : ReplicaMap{};
             for (int q = tid; q < kTile; q += NT) {
                 const int64_t pi = t0 + q;
                 float x = 1e18f, y = 1e18f, z = 1e18f, m = 0.0f, e2 = 0.0f;
                 if (pi < p1) {
                     const int4 pr = f.part[pi];
-                    long long qq[3] = {pr.x, pr.y, pr.z};
-                    if (REPL) replica_q(f, j, pr.x, pr.y, pr.z, qq);
-                    x = (float)(qq[0] - ax) * dlt;
-                    y = (float)(qq[1] - ay) * dlt;
-                    z = (float)(qq[2] - az) * dlt;
+                    int qq[3] = {pr.x, pr.y, pr.z};
+                    if (REPL) replica_q(rm, pr.x, pr.y, pr.z, qq);
+                    x = grid_offset(qq[0], ax) * dlt;
+                    y = grid_offset(qq[1], ay) * dlt;
+                    z = grid_offset(qq[2], az) * dlt;
                     m = __int_as_float(pr.w);
                     if (PEPS) e2 = f.eps2[pi];
                 }
@@ -1178,14 +1183,15 @@ __global__ void __launch_bounds__(NT, 1) k_force_bundle1(ForceArgs A, int group)
             ny = -(float)(((A.py[ic] - o[1]) * f.inv_delta - (double)ay) * f.delta);
             nz = -(float)(((A.pz[ic] - o[2]) * f.inv_delta - (double)az) * f.delta);
         }
+        const ReplicaMap rm = REPL ? replica_map(f, j) : ReplicaMap{};
 #pragma unroll
         for (int k = 0; k < kTile / NT; ++k) {
             const int q = k * NT + tid;
             if (q >= cnt) break;
             const int4 pr = part[k];
-            long long qq[3] = {pr.x, pr.y, pr.z};
-            if (REPL) replica_q(f, j, pr.x, pr.y, pr.z, qq);
-            s_p[q] = make_float4((float)(qq[0] - ax) * dlt, (float)(qq[1] - ay) * dlt, (float)(qq[2] - az) * dlt,
+            int qq[3] = {pr.x, pr.y, pr.z};
+            if (REPL) replica_q(rm, pr.x, pr.y, pr.z, qq);
+            s_p[q] = make_float4(grid_offset(qq[0], ax) * dlt, grid_offset(qq[1], ay) * dlt, grid_offset(qq[2], az) * dlt,
                                  __int_as_float(pr.w));
             if (PEPS) s_e[q] = f.eps2[p0 + q];
         }
@@ -1305,14 +1311,15 @@ __global__ void __launch_bounds__(NT) k_force_fp64(ForceArgs A)
         for (int64_t t0 = p0; t0 < p1; t0 += kTile64) {
             const int cnt = ((int)min(p1 - t0, (int64_t)kTile64) + kUnit64 - 1) / kUnit64 * kUnit64;
             __syncthreads();
+            const ReplicaMap rm = REPL ? replica_map(f, j) : ReplicaMap{};
             for (int q = tid; q < cnt; q += NT) {
                 const int64_t pi = t0 + q;
                 double4_16a v = make_double4_16a(1e100, 1e100, 1e100, 0.0);
                 double e2 = 0.0;
                 if (pi < p1) {
                     const int4 pr = f.part[pi];
-                    long long qq[3] = {pr.x, pr.y, pr.z};
-                    if (REPL) replica_q(f, j, pr.x, pr.y, pr.z, qq);
+                    int qq[3] = {pr.x, pr.y, pr.z};
+                    if (REPL) replica_q(rm, pr.x, pr.y, pr.z, qq);
                     v = make_double4_16a((double)(qq[0] - ax) * f.delta, (double)(qq[1] - ay) * f.delta,
                                          (double)(qq[2] - az) * f.delta, f.m64[pi]);
                     if (PEPS) e2 = f.eps2_64[pi];

@@ -236,17 +236,18 @@ __global__ void __launch_bounds__(kMpNT) k_mp_deflect(MPArgs A)
     const float dlt = (float)f.delta;
     for (int64_t t0 = p0; t0 < p1; t0 += kTile) {
         __syncthreads();
+        const ReplicaMap rm = REPL ? replica_map(f, P.rep) : ReplicaMap{};
         for (int qq = tid; qq < kTile; qq += kMpNT) {
             const int64_t pi = t0 + qq;
             float4 v = make_float4(1e18f, 1e18f, 0.f, 0.f);
             if (pi < p1) {
                 const int4 pr = f.part[pi];
-                long long g[3] = {pr.x, pr.y, pr.z};
-                if (REPL) replica_q(f, P.rep, pr.x, pr.y, pr.z, g);
+                int g[3] = {pr.x, pr.y, pr.z};
+                if (REPL) replica_q(rm, pr.x, pr.y, pr.z, g);
                 if (g[2] >= P.qlo && g[2] <= P.qhi) {
                     ++n_on;
-                    v.x = (float)(g[0] - ax) * dlt;
-                    v.y = (float)(g[1] - ay) * dlt;
+                    v.x = grid_offset(g[0], ax) * dlt;
+                    v.y = grid_offset(g[1], ay) * dlt;
                     v.z = __int_as_float(pr.w);
                     v.w = PEPS ? f.eps2[pi] : f.eps2u;
                 }
@@ -384,16 +385,17 @@ __global__ void __launch_bounds__(kMp2NT, NRING <= 4 ? 8 : 4) k_mp_deflect2(MPAr
         const int lane = tid & 31, warp = tid >> 5;
         float4 rec[K];  // x, y, m, eps^2
         unsigned on[K];
+        const ReplicaMap rm = REPL ? replica_map(f, P.rep) : ReplicaMap{};
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int64_t pi = t0 + k * kMp2NT + tid;
             bool in = false;
             if (pi < p1) {
                 const int4 pr = f.part[pi];
-                long long g[3] = {pr.x, pr.y, pr.z};
-                if (REPL) replica_q(f, P.rep, pr.x, pr.y, pr.z, g);
+                int g[3] = {pr.x, pr.y, pr.z};
+                if (REPL) replica_q(rm, pr.x, pr.y, pr.z, g);
                 in = g[2] >= P.qlo && g[2] <= P.qhi;
-                rec[k] = make_float4(-(float)(g[0] - ax) * dlt, -(float)(g[1] - ay) * dlt, __int_as_float(pr.w),
+                rec[k] = make_float4(-grid_offset(g[0], ax) * dlt, -grid_offset(g[1], ay) * dlt, __int_as_float(pr.w),
                                    PEPS ? f.eps2[pi] : f.eps2u);
             }
             on[k] = __ballot_sync(0xffffffffu, in);
@@ -513,13 +515,14 @@ __global__ void __launch_bounds__(kMpNT64) k_mp_deflect64(MPArgs A)
     const int64_t p1 = min(f.n, p0 + A.per_split);
     for (int64_t t0 = p0; t0 < p1; t0 += kTile64) {
         __syncthreads();
+        const ReplicaMap rm = REPL ? replica_map(f, P.rep) : ReplicaMap{};
         for (int qq = tid; qq < kTile64; qq += kMpNT64) {
             const int64_t pi = t0 + qq;
             double4_16a v = make_double4_16a(1e100, 1e100, 0.0, 0.0);
             if (pi < p1) {
                 const int4 pr = f.part[pi];
-                long long g[3] = {pr.x, pr.y, pr.z};
-                if (REPL) replica_q(f, P.rep, pr.x, pr.y, pr.z, g);
+                int g[3] = {pr.x, pr.y, pr.z};
+                if (REPL) replica_q(rm, pr.x, pr.y, pr.z, g);
                 if (g[2] >= P.qlo && g[2] <= P.qhi) {
                     ++n_on;
                     v = make_double4_16a((double)g[0] * f.delta, (double)g[1] * f.delta, f.m64[pi],

@@ -2,8 +2,7 @@
 with shifts and positions at the edges of their ranges and points far outside
 the box (whose offsets need 64 bits), against the oracle's FP64 placement: the
 grid holds these positions exactly, so the FP64 potential agrees to the
-rounding of a sum of n terms, the mixed one to FP32 rounding of the offsets
-(2^-23 of a box length over separations of a box length: 1e-5)."""
+rounding of a sum of n terms."""
 import itertools
 
 import numpy as np
@@ -15,9 +14,8 @@ import oracle
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("precision,tol", [("fp64", 1e-12), ("mixed", 1e-5)])
 @pytest.mark.parametrize("L", [8.0, 142.5, 500.0])
-def test_every_signed_permutation(precision, tol, L):
+def test_every_signed_permutation(L):
     import paper_1110_4894_gb300 as P
     L = inputs.box_length(L)
     rots = []
@@ -39,11 +37,11 @@ def test_every_signed_permutation(precision, tol, L):
     pts = np.stack([g.uniform(-0.5, 0.5, rep.size) * L, g.uniform(-0.5, 0.5, rep.size) * L,
                     (rep + g.random(rep.size)) * L], 1)
     pts[::3] += 3.0 * L * g.choice((-1, 1), (n_rep, 3))  # outside the replica
-    ctx = P.Context(0, precision=P.FP64 if precision == "fp64" else P.MIXED)
+    ctx = P.Context(0, precision=P.FP64)
     soft = 0.05 * L
     ctx.load_particles(0, pos, mass, soft, replicated=True, box_length=L, rot=rot, shift=shift)
     got = ctx.potential(0, pts, rep)
     ctx.close()
     ref = oracle.potential(oracle.MassField(pos, mass, soft, replicated=True, L=L, rot=rot, shift=shift), pts, rep)
     for k in range(4):
-        assert np.max(np.abs(got[:, k] - ref[:, k])) < tol * np.max(np.abs(ref[:, k]))
+        assert np.max(np.abs(got[:, k] - ref[:, k])) < 1e-12 * np.max(np.abs(ref[:, k]))
