@@ -776,8 +776,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_force_bundle2(ForceArgs A)
                                                     (float2 *)A.out, s_a, s_b, s_e, s_hl);
 }
 
-// Two bundles per thread with the ring separations expanded about the
-// central ray.  With d_c = p - r_c and e_k = r_c - r_k the ring ray's
+// Two bundles per thread (b0 + tid and b0 + NT + tid in a full block) with the
+// ring separations expanded about the central ray.  With d_c = p - r_c and e_k = r_c - r_k the ring ray's
 // separation is d_k = d_c + e_k, so
 //   |d_k|^2 + eps^2 = (|d_c|^2 + eps^2) + (2 e_k . d_c + |e_k|^2)
 //   sum m d_k / r_k^3 = sum m d_c / r_k^3 + e_k sum m / r_k^3.
@@ -788,11 +788,15 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_force_bundle2(ForceArgs A)
 // 52 f32x2 operations for 10 interactions (the unexpanded kernel: 56).
 // (Taking 1/r^2 from MUFU rcp instead of rsqrt^2 saves 5 more but was
 // measured 26 % slower: the MUFU pipe then limits.)
+// PACK: a block short of 2 NT bundles pairs them over half as many threads, and
+// the warps left without any only help to stage (cones of 128-1024 bundles: 157
+// -> 148 ms for 48 of them; 1111 bundles of 8 rays: 2 %).  The single-trace
+// kernel of rings of 4 does without: the branch costs its schedule 3-6 %.
 // AHEAD: read the next particle's records one iteration ahead, so that the
 // shared-memory latency overlaps the current particle's arithmetic (s_a and
 // s_b then hold kTile + 1 records).  It pays in the single-trace kernel;
 // the persistent batched kernel runs faster without it.
-template <int NT, int NRING, bool REPL, bool PEPS, bool UMASS, int CL, bool AHEAD = true>
+template <int NT, int NRING, bool REPL, bool PEPS, bool UMASS, int CL, bool AHEAD, bool PACK>
 __device__ __forceinline__ void bundle2x_block_sum(const DevField &f, const double *__restrict__ px,
                                                    const double *__restrict__ py, const double *__restrict__ pz,
                                                    const int *__restrict__ rep, int64_t n_b, int64_t n_rays,
@@ -803,8 +807,11 @@ __device__ __forceinline__ void bundle2x_block_sum(const DevField &f, const doub
     constexpr int NR = NRING + 1;
     constexpr int NQ = NR * 3 + NRING;  // compensated sums per bundle: G (3 per ray) and S (ring)
     const int tid = threadIdx.x;
-    int64_t bb[2] = {b0 + tid, b0 + NT + tid};
-    bool valid[2] = {bb[0] < n_b, bb[1] < n_b};
+    static_assert(!PACK || CL == 1, "a cluster's blocks pair their bundles alike");
+    const int half = PACK ? (int)min((int64_t)NT, (n_b - b0 + 1) / 2) : NT;
+    int64_t bb[2] = {b0 + tid, b0 + half + tid};
+    bool valid[2] = {tid < half && bb[0] < n_b, tid < half && bb[1] < n_b};
+    const bool idle = (tid & ~31) >= half;
     __shared__ int s_rmin, s_rmax;
     if (tid == 0) {
         s_rmin = INT_MAX;
@@ -890,6 +897,7 @@ __device__ __forceinline__ void bundle2x_block_sum(const DevField &f, const doub
                 if (PEPS) s_e[q] = e2;
             }
             __syncthreads();
+            if (PACK && idle) continue;
             for (int c0 = 0; c0 < kTile; c0 += kChunk2) {
                 float2 cx[NR], cy[NR], cz[NR], cs[NRING];
 #pragma unroll
@@ -1103,7 +1111,7 @@ __global__ void __launch_bounds__(NT, TPSM / NT) k_force_bundle2x(ForceArgs A)
     const int split = blockIdx.y;
     const int64_t p0 = (int64_t)split * A.per_split;
     const int64_t p1 = min(A.f.n, p0 + A.per_split);
-    bundle2x_block_sum<NT, NRING, REPL, PEPS, UMASS, CL, AHEAD>(A.f, A.px, A.py, A.pz, A.rep, n_b, A.n, b0, p0, p1,
+    bundle2x_block_sum<NT, NRING, REPL, PEPS, UMASS, CL, AHEAD, NRING == 8>(A.f, A.px, A.py, A.pz, A.rep, n_b, A.n, b0, p0, p1,
                                                             split, (float2 *)A.out, s_a, s_b, s_e, s_hl);
 }
 
