@@ -74,10 +74,13 @@ cudaError_t launch_init(const TraceParams &tp, const DevField &f, const double *
 // (reduce_step), then one warp runs the FP64 stage update of the 32 rays.  The
 // sum is a chain of thousands of steps in few warps where few bundles meet many
 // particles (4096 splits of 640 rays: 281 us a stage while its loads waited for
-// one another), so kAhead rows of partials are kept in flight in registers (84
-// us).
+// one another), so AHEAD rows of partials are kept in flight in registers: 84 us
+// with 64 rows.  96 rows leave an SM two blocks instead of three, so they serve
+// the launches that give no SM two (76 us; a whole stage of 128 bundles in the
+// 1048576-particle box 457.4 -> 449.5 us, but of 4096 bundles and 196 splits 848
+// -> 861 us).
 constexpr int kStageRays = 32, kStageThreads = 4 * kStageRays;
-constexpr int kRows = 16, kAhead = 64;  // rows per load group, rows in flight
+constexpr int kRows = 16;  // rows per load group
 // from this many rays on (four blocks of 256 per SM), one ray per thread
 // still gives every SM several blocks
 static int64_t stage_wide_rays() { return (int64_t)device_sm_count() * 4 * 256; }
@@ -120,6 +123,7 @@ cudaError_t launch_prism(const TraceParams &tp, const DevField &f, RayState rs, 
                              d_counters, d_prism);
 }
 
+template <int AHEAD>
 __global__ void __launch_bounds__(kStageThreads) k_stage(TraceParams tp, DevField f, RayState rs, int S, int fp64,
                                                         double mfac, const float2 *partials,
                                                         const double *dlam,
@@ -134,7 +138,7 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(TraceParams tp, DevFiel
     const int o = threadIdx.x / kStageRays, lane = threadIdx.x % kStageRays;
     const int64_t i = (int64_t)blockIdx.x * kStageRays + lane;
     if (i < rs.n_rays) {
-        constexpr int G = kAhead / kRows;
+        constexpr int G = AHEAD / kRows;
         const float2 *src = partials + (int64_t)o * rs.n_rays + i;
         const int64_t pitch = 4 * rs.n_rays;
         float2 buf[G][kRows];
@@ -148,7 +152,7 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(TraceParams tp, DevFiel
         for (int g = 0; g < G; ++g) load(g, g * kRows);
         float hi = 0.0f, lo = 0.0f;
         double acc = 0.0;
-        for (int s0 = 0; s0 < S; s0 += kAhead) {
+        for (int s0 = 0; s0 < S; s0 += AHEAD) {
 #pragma unroll
             for (int g = 0; g < G; ++g) {
                 if (s0 + g * kRows >= S) break;
@@ -160,7 +164,7 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(TraceParams tp, DevFiel
 #pragma unroll
                     for (int r = 0; r < kRows; ++r) reduce_step(hi, lo, buf[g][r]);
                 }
-                load(g, s0 + kAhead + g * kRows);
+                load(g, s0 + AHEAD + g * kRows);
             }
         }
         s_acc[lane][o] = fp64 ? acc : (double)hi + (double)lo;
@@ -220,7 +224,8 @@ cudaError_t launch_stage(const TraceParams &tp, const DevField &f, RayState rs, 
                                  d_partials, d_dlam, d_misc, step, stage, d_counters, d_prism);
     } else {
         const int64_t blocks = (rs.n_rays + kStageRays - 1) / kStageRays;
-        return launch_overlapped(k_stage, dim3((unsigned)blocks), kStageThreads, st, tp, f, rs, S, fp64 ? 1 : 0, mfac,
+        return launch_overlapped(blocks <= device_sm_count() ? k_stage<96> : k_stage<64>, dim3((unsigned)blocks),
+                                 kStageThreads, st, tp, f, rs, S, fp64 ? 1 : 0, mfac,
                                  (const float2 *)d_partials, d_dlam, d_misc, step, stage, d_counters, d_prism);
     }
 }

@@ -29,3 +29,23 @@ def test_any_number_of_splits(precision, bundles):
         ctx.close()
     for r in res[1:]:
         assert np.max(np.abs(r - res[0])) <= 1e-9 * np.max(np.abs(res[0]))
+
+
+# (40 bundles give no SM two of the stage's blocks of 32 rays, 1100 do: 96 and 64
+# rows in flight)
+@pytest.mark.parametrize("bundles", [40, 1100])
+def test_splits_around_the_rows_in_flight(bundles):
+    import paper_1110_4894_gb300 as P
+    n = 256 * 130
+    g = inputs.rng(inputs.BASE_SEED + 131)
+    pos = inputs.quantize(np.array([0.0, 0.0, 1000.0]) + 0.5 * g.normal(size=(n, 3)))
+    theta = np.array([3e-4, -2e-4]) + 2e-4 * g.normal(size=(bundles, 2))
+    res = []
+    for splits in (9, 63, 64, 65, 95, 96, 97, 130):
+        ctx = P.Context(0, precision=P.MIXED, splits=splits)
+        ctx.set_cosmology(0.3, 0.7, 0.7)
+        ctx.load_particles(0, pos, 1e9, 0.05)
+        res.append(ctx.trace(0, 0.5, theta, n_ring=4, theta_r=5e-6, n_steps=6)["mu"])
+        ctx.close()
+    for r in res[1:]:
+        assert np.max(np.abs(r - res[0])) <= 1e-9 * np.max(np.abs(res[0]))
