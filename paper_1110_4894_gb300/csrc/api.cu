@@ -1126,7 +1126,7 @@ static int trace_advance(rt3d_ctx *ctx, int n, cudaStream_t st)
         }
         CK(launch_stage(T.tp, fs.df, T.rs, T.sh, T.fp64, s.partials, s.dlam, s.misc, step, stage, s.counters, st,
                         T.use_prism ? s.prism : nullptr));
-        T.launches += 2;
+        T.launches += 2 + stage_merges(T.sh, T.fp64, n_rays);
         T.flaunch += gate ? 0 : 1;
     }
     ctx->stats.launches = T.launches;

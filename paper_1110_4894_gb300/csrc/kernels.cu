@@ -123,6 +123,118 @@ cudaError_t launch_prism(const TraceParams &tp, const DevField &f, RayState rs, 
                              d_counters, d_prism);
 }
 
+// The sum of many split partials ahead of the stage, in place: row 0 of the
+// partials becomes the double-float sum of all rows, the same bits as k_stage's
+// own sum.  There a warp issues some twelve instructions a row, and few rays make
+// few warps (640 rays x 4096 splits: 80 warps on 20 SMs, 72 us).  Only the
+// additions hi + x and lo + w are chains: here one warp runs both (lanes 0-15 the
+// high sums of tile k of kMergeRows rows, lanes 16-31 the low sums of tile
+// k - 2), and the other warps do what is not serial in between: the TwoSum errors
+// w of tile k - 1, and the copies of later tiles into shared memory.  16 rays of
+// one output a block (a row is then a 128-byte line), so 640 rays use every SM:
+// 38 us.  What is left is the chain, 16 cycles a row with a tile's barrier; more
+// tiles in flight, longer ones, or more helper warps change nothing.
+constexpr int kMergeRays = 16, kMergeRows = 48, kMergeTiles = 6, kMergeHelpers = 192, kMergeThreads = 32 + kMergeHelpers;
+constexpr int kMergeAhead = kMergeTiles - 3;  // tiles on their way; three are in use
+constexpr int kMergeGroup = 16;               // rows that the chains read ahead of their additions
+// From 256 rows on, and up to two blocks an SM.  A whole stage (k_stage alone ->
+// with k_merge, us): 64 bundles and 65,536 particles (256 splits) 171 -> 141, 64
+// bundles and 1,048,576 particles 551 -> 526, 128 of 5 rays 449 -> 429, 128 of 9
+// rays (288 blocks) 835 -> 807; but 256 of 5 rays (320 blocks, and warps enough
+// for k_stage) 737 -> 746, 768 of 5 3692 -> 3714, and 200 bundles with 118 splits
+// 50 -> 53.
+constexpr int kMergeFrom = 256;
+static int64_t merge_blocks(int64_t n_rays) { return (n_rays + kMergeRays - 1) / kMergeRays; }
+bool stage_merges(const ForceShape &sh, bool fp64, int64_t n_rays)
+{
+    return !fp64 && partial_splits(sh) >= kMergeFrom && 4 * merge_blocks(n_rays) <= 2 * (int64_t)device_sm_count();
+}
+
+__device__ __forceinline__ void copy_async8(void *dst, const void *src, bool valid)  // zeros if not valid
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(valid ? 8 : 0)
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(kMergeThreads) k_merge(float2 *partials, int S, int64_t n_rays, int n_steps, int step,
+                                                         const unsigned long long *cnt)
+{
+    __shared__ float2 s_v[kMergeTiles][kMergeRows][kMergeRays];  // (x, y) of a row; y becomes w
+    __shared__ float s_t[2][kMergeRows + 1][kMergeRays];         // high sums before each row, and after the last
+    let_next_start();
+    wait_for_previous();
+    if (step >= n_steps && cnt[(step - 1) & 1] == 0ull) return;  // every ray is across
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, o = blockIdx.y;
+    const int64_t i0 = (int64_t)blockIdx.x * kMergeRays;
+    const int n_tiles = (S + kMergeRows - 1) / kMergeRows;
+    const int r = lane % kMergeRays;
+    // a helper thread has ray r of every kStep-th row, from row0 on
+    constexpr int kStep = kMergeHelpers / kMergeRays, kEach = kMergeRows / kStep;
+    static_assert(kEach * kStep == kMergeRows, "whole rows per helper thread");
+    const int row0 = ((int)threadIdx.x - 32) / kMergeRays;
+    const float2 *src = partials + ((int64_t)row0 * 4 + o) * n_rays + i0 + r;
+    const int64_t pitch = (int64_t)kStep * 4 * n_rays;
+    int stage_in = 0, left = i0 + r < n_rays ? S - row0 : 0;  // slot of the next tile; rows of this thread's from here
+    const auto load = [&]() {
+#pragma unroll
+        for (int j = 0; j < kEach; ++j, left -= kStep, src += pitch)
+            copy_async8(&s_v[stage_in][row0 + j * kStep][r], left > 0 ? src : partials, left > 0);
+        stage_in = stage_in + 1 == kMergeTiles ? 0 : stage_in + 1;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (warp > 0)
+        for (int t = 0; t < kMergeAhead; ++t) load();
+    const bool high = lane < kMergeRays;
+    float acc = 0.0f;  // of this lane's chain
+    for (int k = 0; k < n_tiles + 2; ++k) {
+        if (warp > 0) asm volatile("cp.async.wait_group %0;" ::"n"(kMergeAhead - 1) : "memory");  // tile k is there
+        __syncthreads();
+        if (warp == 0) {
+            const int t = high ? k : k - 2;
+            if (t >= 0 && t < n_tiles) {
+                const float *src = high ? &s_v[t % kMergeTiles][0][r].x : &s_v[t % kMergeTiles][0][r].y;
+                float *dst = &s_t[t & 1][0][r];
+                float v[2][kMergeGroup];
+#pragma unroll
+                for (int q = 0; q < kMergeGroup; ++q) v[0][q] = src[q * 2 * kMergeRays];
+#pragma unroll
+                for (int g = 0; g < kMergeRows / kMergeGroup; ++g) {
+                    if (g + 1 < kMergeRows / kMergeGroup) {
+#pragma unroll
+                        for (int q = 0; q < kMergeGroup; ++q)
+                            v[(g + 1) & 1][q] = src[((g + 1) * kMergeGroup + q) * 2 * kMergeRays];
+                    }
+#pragma unroll
+                    for (int q = 0; q < kMergeGroup; ++q) {
+                        if (high) dst[(g * kMergeGroup + q) * kMergeRays] = acc;
+                        acc += v[g & 1][q];
+                    }
+                }
+                if (high) dst[kMergeRows * kMergeRays] = acc;
+            }
+        } else {
+            load();
+            if (k >= 1 && k <= n_tiles) {
+                const int t = k - 1;
+                float2(*tile)[kMergeRays] = s_v[t % kMergeTiles];
+                float(*sums)[kMergeRays] = s_t[t & 1];
+#pragma unroll
+                for (int j = 0; j < kEach; ++j) {
+                    const int row = row0 + j * kStep;
+                    const float hi = sums[row][r], sum = sums[row + 1][r];
+                    const float2 v = tile[row][r];
+                    const float bb = sum - hi;
+                    tile[row][r].y = (hi - (sum - bb)) + (v.x - bb) + v.y;
+                }
+            }
+        }
+    }
+    if (warp > 0) return;
+    const float lo = __shfl_down_sync(0xffffffffu, acc, kMergeRays);
+    if (high && i0 + r < n_rays) partials[o * n_rays + i0 + r] = make_float2(acc, lo);
+}
+
 template <int AHEAD>
 __global__ void __launch_bounds__(kStageThreads) k_stage(TraceParams tp, DevField f, RayState rs, int S, int fp64,
                                                         double mfac, const float2 *partials,
@@ -209,7 +321,7 @@ __global__ void __launch_bounds__(256) k_stage_wide(TraceParams tp, DevField f, 
 }
 
 cudaError_t launch_stage(const TraceParams &tp, const DevField &f, RayState rs, const ForceShape &sh, bool fp64,
-                         const void *d_partials, const double *d_dlam, const double *d_misc, int step, int stage,
+                         void *d_partials, const double *d_dlam, const double *d_misc, int step, int stage,
                          unsigned long long *d_counters, cudaStream_t st, const double *d_prism)
 {
     const int S = partial_splits(sh);
@@ -224,6 +336,14 @@ cudaError_t launch_stage(const TraceParams &tp, const DevField &f, RayState rs, 
                                  d_partials, d_dlam, d_misc, step, stage, d_counters, d_prism);
     } else {
         const int64_t blocks = (rs.n_rays + kStageRays - 1) / kStageRays;
+        if (stage_merges(sh, fp64, rs.n_rays)) {
+            const cudaError_t e = launch_overlapped(k_merge, dim3((unsigned)merge_blocks(rs.n_rays), 4), kMergeThreads,
+                                                    st, (float2 *)d_partials, S, rs.n_rays, tp.n_steps, step,
+                                                    d_counters);
+            if (e != cudaSuccess) return e;
+            return launch_overlapped(k_stage<16>, dim3((unsigned)blocks), kStageThreads, st, tp, f, rs, 1, 0, mfac,
+                                     (const float2 *)d_partials, d_dlam, d_misc, step, stage, d_counters, d_prism);
+        }
         return launch_overlapped(blocks <= device_sm_count() ? k_stage<96> : k_stage<64>, dim3((unsigned)blocks),
                                  kStageThreads, st, tp, f, rs, S, fp64 ? 1 : 0, mfac,
                                  (const float2 *)d_partials, d_dlam, d_misc, step, stage, d_counters, d_prism);

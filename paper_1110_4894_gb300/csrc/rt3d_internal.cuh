@@ -418,9 +418,11 @@ cudaError_t launch_init(const TraceParams &tp, const DevField &f, const double *
 cudaError_t launch_force(const DevField &f, const RayState &rs, const ForceShape &sh, bool fp64,
                          void *d_partials, const unsigned long long *d_active, int gate, cudaStream_t st);
 cudaError_t launch_stage(const TraceParams &tp, const DevField &f, RayState rs, const ForceShape &sh,
-                         bool fp64, const void *d_partials, const double *d_dlam, const double *d_misc,
+                         bool fp64, void *d_partials, const double *d_dlam, const double *d_misc,
                          int step, int stage, unsigned long long *d_counters, cudaStream_t st,
                          const double *d_prism = nullptr);
+// whether launch_stage adds the split partials up in a kernel of its own first
+bool stage_merges(const ForceShape &sh, bool fp64, int64_t n_rays);
 // per-bundle prism records (value, gradient, Hessian at the central ray) of a
 // mean-subtracted replicated field, for launch_stage: kPrismRec doubles each
 constexpr int kPrismRec = 13;

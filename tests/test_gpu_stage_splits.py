@@ -49,3 +49,23 @@ def test_splits_around_the_rows_in_flight(bundles):
         ctx.close()
     for r in res[1:]:
         assert np.max(np.abs(r - res[0])) <= 1e-9 * np.max(np.abs(res[0]))
+
+
+# (from 256 splits on, and up to 4864 / 4 rays, a kernel of its own adds the
+# partials up, in tiles of 48 rows and blocks of 16 rays)
+@pytest.mark.parametrize("bundles,n_ring", [(1, 4), (3, 4), (16, 8), (33, 4), (130, 8), (243, 4)])
+@pytest.mark.parametrize("splits", [256, 287, 288, 289, 480, 700])
+def test_many_splits(bundles, n_ring, splits):
+    import paper_1110_4894_gb300 as P
+    n = 256 * splits - 3
+    g = inputs.rng(inputs.BASE_SEED + 132)
+    pos = inputs.quantize(np.array([0.0, 0.0, 1000.0]) + 0.5 * g.normal(size=(n, 3)))
+    theta = np.array([3e-4, -2e-4]) + 2e-4 * g.normal(size=(bundles, 2))
+    res = []
+    for s in (64, splits):
+        ctx = P.Context(0, precision=P.MIXED, splits=s)
+        ctx.set_cosmology(0.3, 0.7, 0.7)
+        ctx.load_particles(0, pos, 1e9 * 33280 / n, 0.05)
+        res.append(ctx.trace(0, 0.5, theta, n_ring=n_ring, theta_r=5e-6, n_steps=6)["mu"])
+        ctx.close()
+    assert np.max(np.abs(res[1] - res[0])) <= 1e-9 * np.max(np.abs(res[0]))
