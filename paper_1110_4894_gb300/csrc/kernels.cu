@@ -75,10 +75,10 @@ cudaError_t launch_init(const TraceParams &tp, const DevField &f, const double *
 // sum is a chain of thousands of steps in few warps where few bundles meet many
 // particles (4096 splits of 640 rays: 281 us a stage while its loads waited for
 // one another), so AHEAD rows of partials are kept in flight in registers: 84 us
-// with 64 rows.  96 rows leave an SM two blocks instead of three, so they serve
-// the launches that give no SM two (76 us; a whole stage of 128 bundles in the
-// 1048576-particle box 457.4 -> 449.5 us, but of 4096 bundles and 196 splits 848
-// -> 861 us).
+// with 64 rows.  96 rows leave an SM two blocks instead of three and pay off over
+// many splits where the launch gives no SM two (a whole stage of 256 bundles in
+// the 1,048,576-particle box, 2048 splits: 744 -> 734 us; but 200 bundles and 118
+// splits 47.7 -> 48.4, 4096 bundles and 196 splits 848 -> 861).
 constexpr int kStageRays = 32, kStageThreads = 4 * kStageRays;
 constexpr int kRows = 16;  // rows per load group
 // from this many rays on (four blocks of 256 per SM), one ray per thread
@@ -137,7 +137,7 @@ cudaError_t launch_prism(const TraceParams &tp, const DevField &f, RayState rs, 
 constexpr int kMergeRays = 16, kMergeRows = 48, kMergeTiles = 6, kMergeHelpers = 192, kMergeThreads = 32 + kMergeHelpers;
 constexpr int kMergeAhead = kMergeTiles - 3;  // tiles on their way; three are in use
 constexpr int kMergeGroup = 16;               // rows that the chains read ahead of their additions
-// From 256 rows on, and up to two blocks an SM.  A whole stage (k_stage alone ->
+// Many splits: from 256 rows on; k_merge up to two of its blocks an SM.  A whole stage (k_stage alone ->
 // with k_merge, us): 64 bundles and 65,536 particles (256 splits) 171 -> 141, 64
 // bundles and 1,048,576 particles 551 -> 526, 128 of 5 rays 449 -> 429, 128 of 9
 // rays (288 blocks) 835 -> 807; but 256 of 5 rays (320 blocks, and warps enough
@@ -344,7 +344,7 @@ cudaError_t launch_stage(const TraceParams &tp, const DevField &f, RayState rs, 
             return launch_overlapped(k_stage<16>, dim3((unsigned)blocks), kStageThreads, st, tp, f, rs, 1, 0, mfac,
                                      (const float2 *)d_partials, d_dlam, d_misc, step, stage, d_counters, d_prism);
         }
-        return launch_overlapped(blocks <= device_sm_count() ? k_stage<96> : k_stage<64>, dim3((unsigned)blocks),
+        return launch_overlapped(S >= kMergeFrom && blocks <= device_sm_count() ? k_stage<96> : k_stage<64>, dim3((unsigned)blocks),
                                  kStageThreads, st, tp, f, rs, S, fp64 ? 1 : 0, mfac,
                                  (const float2 *)d_partials, d_dlam, d_misc, step, stage, d_counters, d_prism);
     }
