@@ -137,12 +137,12 @@ cudaError_t launch_prism(const TraceParams &tp, const DevField &f, RayState rs, 
 constexpr int kMergeRays = 16, kMergeRows = 48, kMergeTiles = 6, kMergeHelpers = 192, kMergeThreads = 32 + kMergeHelpers;
 constexpr int kMergeAhead = kMergeTiles - 3;  // tiles on their way; three are in use
 constexpr int kMergeGroup = 16;               // rows that the chains read ahead of their additions
-// Many splits: from 256 rows on; k_merge up to two of its blocks an SM.  A whole stage (k_stage alone ->
-// with k_merge, us): 64 bundles and 65,536 particles (256 splits) 171 -> 141, 64
-// bundles and 1,048,576 particles 551 -> 526, 128 of 5 rays 449 -> 429, 128 of 9
-// rays (288 blocks) 835 -> 807; but 256 of 5 rays (320 blocks, and warps enough
-// for k_stage) 737 -> 746, 768 of 5 3692 -> 3714, and 200 bundles with 118 splits
-// 50 -> 53.
+// Many splits: from 256 rows on.  k_merge up to two of its blocks an SM; a whole
+// stage (k_stage alone -> with k_merge, us): 64 bundles and 65,536 particles (256
+// splits) 171 -> 141, 64 bundles and 1,048,576 particles 551 -> 526, 128 of 5 rays
+// 449 -> 429, 128 of 9 rays (288 blocks) 835 -> 807; but 256 of 5 rays (320
+// blocks, and warps enough for k_stage) 737 -> 746, 768 of 5 3692 -> 3714, and 200
+// bundles with 118 splits 50 -> 53.
 constexpr int kMergeFrom = 256;
 static int64_t merge_blocks(int64_t n_rays) { return (n_rays + kMergeRays - 1) / kMergeRays; }
 bool stage_merges(const ForceShape &sh, bool fp64, int64_t n_rays)
@@ -230,7 +230,10 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge(float2 *partials, int S
             }
         }
     }
-    if (warp > 0) return;
+    if (warp > 0) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        return;
+    }
     const float lo = __shfl_down_sync(0xffffffffu, acc, kMergeRays);
     if (high && i0 + r < n_rays) partials[o * n_rays + i0 + r] = make_float2(acc, lo);
 }
@@ -254,11 +257,13 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(TraceParams tp, DevFiel
         const float2 *src = partials + (int64_t)o * rs.n_rays + i;
         const int64_t pitch = 4 * rs.n_rays;
         float2 buf[G][kRows];
-        // (rows past the last split are zeros, which leave the sum as it is)
+        // (rows past the last split are zeros, which leave the sum as it is; read
+        // from L2: this block may have started while k_merge, on the same SM, had
+        // the lines of row 0 in L1)
         const auto load = [&](int g, int s0) {
 #pragma unroll
             for (int r = 0; r < kRows; ++r, src += pitch)
-                buf[g][r] = s0 + r < S ? __ldg(src) : make_float2(0.0f, 0.0f);
+                buf[g][r] = s0 + r < S ? __ldcg(src) : make_float2(0.0f, 0.0f);
         };
 #pragma unroll
         for (int g = 0; g < G; ++g) load(g, g * kRows);
@@ -344,8 +349,8 @@ cudaError_t launch_stage(const TraceParams &tp, const DevField &f, RayState rs, 
             return launch_overlapped(k_stage<16>, dim3((unsigned)blocks), kStageThreads, st, tp, f, rs, 1, 0, mfac,
                                      (const float2 *)d_partials, d_dlam, d_misc, step, stage, d_counters, d_prism);
         }
-        return launch_overlapped(S >= kMergeFrom && blocks <= device_sm_count() ? k_stage<96> : k_stage<64>, dim3((unsigned)blocks),
-                                 kStageThreads, st, tp, f, rs, S, fp64 ? 1 : 0, mfac,
+        return launch_overlapped(S >= kMergeFrom && blocks <= device_sm_count() ? k_stage<96> : k_stage<64>,
+                                 dim3((unsigned)blocks), kStageThreads, st, tp, f, rs, S, fp64 ? 1 : 0, mfac,
                                  (const float2 *)d_partials, d_dlam, d_misc, step, stage, d_counters, d_prism);
     }
 }
