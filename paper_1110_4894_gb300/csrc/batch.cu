@@ -169,8 +169,9 @@ __device__ __noinline__ void batch_grid_item(const BatchCone &C, int rb, int RB,
     }
 }
 
-// the next item: cone, phase and index; cone -1 when all cones are done (or the
-// watchdog expired).  A whole warp calls this.
+// the next item: cone, phase and index; cone -1 when all cones are done or the
+// watchdog expired in any block (looked for before every item, so that such a
+// launch ends with the items in hand).  A whole warp calls this.
 struct BatchWork {
     int cone;
     unsigned phase, item;
@@ -181,6 +182,10 @@ __device__ __forceinline__ void take_work(const BatchArgs &B, BatchWork *w)
     const int lane = threadIdx.x & 31;
     for (;;) {
         const unsigned event = *(volatile unsigned *)(B.bar + 1);  // before looking: what opens later changes it
+        if (__any_sync(0xffffffffu, *(volatile int *)B.err != 0)) {
+            if (lane == 0) *w = BatchWork{-1, 0u, 0u};
+            return;
+        }
         for (int base = 0; base < B.n_cones; base += 32) {
             const int c = base + lane < B.n_cones ? B.order[base + lane] : -1;
             bool some = false;
@@ -208,7 +213,7 @@ __device__ __forceinline__ void take_work(const BatchArgs &B, BatchWork *w)
         }
         int stop = 0;
         if (lane == 0) {
-            stop = *(volatile unsigned *)B.bar >= (unsigned)B.n_cones || *(volatile int *)B.err != 0;
+            stop = *(volatile unsigned *)B.bar >= (unsigned)B.n_cones;
             if (!stop) stop = !bounded_wait(B.bar + 1, event, B.err, B.limit_ns);
             if (stop) *w = BatchWork{-1, 0u, 0u};
         }
