@@ -319,15 +319,32 @@ __device__ __forceinline__ int replica_of(const DevField &f, double x3)
 // 1 / sqrt(x) of a positive FP64 number: the hardware's approximation y
 // (rsqrt.approx.ftz.f64, relative error 2^-20 or better, its low word zero, so
 // y^2 is exact), corrected by the binomial series (1 - e)^(-1/2) = 1 + e / 2 + 3
-// e^2 / 8 + ... for e = 1 - x y^2; the term left out is below 2^-61.  Five FP64
-// operations, no branch.  x = 0 gives infinity, as rsqrt does.
-__device__ __forceinline__ double rsqrt_series(double x)
+// e^2 / 8 + ... for e = 1 - x y^2; |e| <= 2^-19, so the term left out, 5 e^3 / 16,
+// is below 2^-58.  Five FP64 operations, where x and y^2 are normal numbers.
+// Subnormal numbers and those from 2^1022 on are scaled by a power of two first;
+// zero gives infinity, infinity zero and NaN NaN, as rsqrt does.
+__device__ __forceinline__ double rsqrt_estimate(double x)
 {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y * y, 1.0), t = e * fma(e, 0.375, 0.5);
-    const double r = fma(y, t, y);
-    return __double2hiint(y) == 0x7ff00000 ? y : r;  // x = 0 (an integer compare)
+    return y;
+}
+
+__device__ __forceinline__ double rsqrt_corrected(double x, double y)
+{
+    const double e = fma(-x, y * y, 1.0);
+    return fma(y, e * fma(e, 0.375, 0.5), y);
+}
+
+__device__ __forceinline__ double rsqrt_series(double x)
+{
+    if ((unsigned)__double2hiint(x) - 0x00100000u >= 0x7fc00000u) {
+        const bool small = __double2hiint(x) < 0x00100000;
+        x *= small ? 0x1p108 : 0x1p-108;
+        const double y = rsqrt_estimate(x);
+        return y > 0.0 && y < 0x1p1000 ? rsqrt_corrected(x, y) * (small ? 0x1p54 : 0x1p-54) : y;
+    }
+    return rsqrt_corrected(x, rsqrt_estimate(x));
 }
 
 // one particle of mass m at offset d: adds m / r and m d / r^3, r^2 = |d|^2 + e2
