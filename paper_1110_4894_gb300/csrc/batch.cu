@@ -181,7 +181,9 @@ __device__ __forceinline__ void take_work(const BatchArgs &B, BatchWork *w)
 {
     const int lane = threadIdx.x & 31;
     for (;;) {
-        const unsigned event = *(volatile unsigned *)(B.bar + 1);  // before looking: what opens later changes it
+        __syncwarp();  // lane 0 may come from opening a phase: no lane looks before it has
+        const unsigned event = *(volatile unsigned *)(B.bar + 1);
+        __threadfence();  // read before looking: what opens later changes it
         if (__any_sync(0xffffffffu, *(volatile int *)B.err != 0)) {
             if (lane == 0) *w = BatchWork{-1, 0u, 0u};
             return;

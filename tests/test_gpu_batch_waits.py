@@ -44,3 +44,23 @@ def test_expired_watchdog_ends_the_launch():
     for k, v in ctx.trace_batch(short, **kw)[0].items():
         assert np.array_equal(v, ref[k]), k
     ctx.close()
+
+
+@pytest.mark.parametrize("cones", [1, 2, 33])
+def test_no_block_sleeps_through_a_phase(cones):
+    """cones of one force item and one stage item: each phase is opened by the block that ran the one before, and
+    whoever finds no work has to wake when it opens.  4000 phases a cone under a limit that one missed wake-up of
+    the last waiting block would exceed."""
+    import paper_1110_4894_gb300 as P
+    theta = 4e-4 * inputs.rng(3).normal(size=(5, 2))
+    kw = dict(n_ring=4, theta_r=5e-6)
+    batch = [dict(field_id=0, z_s=0.5, theta=theta, n_steps=500)] * cones
+    ctx = context(P, watchdog_s=0.5)
+    ctx.load_particles(0, inputs.quantize(np.array([[0.0, 0.0, 700.0], [0.1, 0.2, 700.5]])), 5e7, 0.3)
+    runs = [ctx.trace_batch(batch, **kw) for _ in range(3)]
+    one = ctx.trace(0, 0.5, theta, n_steps=500, **kw)
+    ctx.close()
+    for run in runs:
+        for out in run:
+            assert np.array_equal(out["mu"], runs[0][0]["mu"])
+    assert np.max(np.abs(runs[0][0]["mu"] / one["mu"] - 1)) < 1e-6
