@@ -508,7 +508,6 @@ struct Builder {
     double h = 0.0, eps2 = 0.0;
     bool keep = false, have_k = false;
     double *pos = nullptr, *mass = nullptr, *buf = nullptr, *val = nullptr, *y2 = nullptr;
-    int64_t cap = 0;
     unsigned long long *q = nullptr, *total = nullptr;
     cufftDoubleComplex *fm = nullptr, *fk = nullptr, *kspec = nullptr;
     cufftHandle r2c = 0, c2r = 0, c2c = 0;  // half the planes, both ways; along x1
@@ -557,7 +556,8 @@ struct Builder {
         if (r_ != CUFFT_SUCCESS) return B.fft_fail(r_, what); \
     } while (0)
 
-static int builder_init(Builder &B, int n, double h, double soft, cudaStream_t st, std::string &err)
+// np_most: the most particles of any grid to be built
+static int builder_init(Builder &B, int n, double h, double soft, int64_t np_most, cudaStream_t st, std::string &err)
 {
     B.n = n;
     B.h = h;
@@ -571,6 +571,10 @@ static int builder_init(Builder &B, int n, double h, double soft, cudaStream_t s
     GCK(cudaMalloc(&B.fk, sizeof(cufftDoubleComplex) * (size_t)B.Pc()), "grid FFT buffer");
     GCK(cudaMalloc(&B.val, sizeof(double) * 4 * (size_t)B.n3()), "grid values");
     GCK(cudaMalloc(&B.y2, sizeof(double) * 4 * (size_t)B.n3()), "grid spline table");
+    if (np_most > 0) {
+        GCK(cudaMalloc(&B.pos, sizeof(double) * 3 * (size_t)np_most), "particle upload");
+        GCK(cudaMalloc(&B.mass, sizeof(double) * (size_t)np_most), "particle upload");
+    }
     int plane[2] = {P, P}, half[2] = {P, n + 1}, line[1] = {P};
     const int pd = P * P, pc = P * (n + 1);
     FCK(cufftPlanMany(&B.r2c, 2, plane, plane, 1, pd, half, 1, pc, CUFFT_D2Z, n), "cufftPlanMany D2Z");
@@ -582,14 +586,20 @@ static int builder_init(Builder &B, int n, double h, double soft, cudaStream_t s
     FCK(cufftSetStream(B.r2c, st), "cufftSetStream");
     FCK(cufftSetStream(B.c2r, st), "cufftSetStream");
     FCK(cufftSetStream(B.c2c, st), "cufftSetStream");
-    // the two kernel spectra stay resident where they are small and fit
-    B.keep = 2 * B.Pc() * (int64_t)sizeof(cufftDoubleComplex) <= ((int64_t)8 << 30);
-    if (B.keep && cudaMalloc(&B.kspec, sizeof(cufftDoubleComplex) * 2 * (size_t)B.Pc()) != cudaSuccess) {
+    return RT3D_OK;
+}
+
+// The two kernel spectra stay resident where they are small and fit.  Called
+// after everything that a build cannot do without has its memory.
+static void builder_keep_spectra(Builder &B)
+{
+    const size_t bytes = 2 * (size_t)B.Pc() * sizeof(cufftDoubleComplex);
+    B.keep = bytes <= ((size_t)8 << 30);
+    if (B.keep && cudaMalloc(&B.kspec, bytes) != cudaSuccess) {
         cudaGetLastError();
         B.kspec = nullptr;
         B.keep = false;
     }
-    return RT3D_OK;
 }
 
 // one grid: the particles' CIC node masses on the nodes lo + h i, optionally
@@ -608,16 +618,6 @@ static int builder_run(Builder &B, int64_t np, const double *pos, const double *
     GCK(cudaMemsetAsync(B.q, 0, sizeof(unsigned long long) * (size_t)n3, st), "memset");
     GCK(cudaMemsetAsync(B.total, 0, sizeof(unsigned long long), st), "memset");
     if (np > 0) {
-        if (np > B.cap) {
-            GCK(cudaStreamSynchronize(st), "grid build");
-            cudaFree(B.pos);
-            cudaFree(B.mass);
-            B.pos = B.mass = nullptr;
-            B.cap = 0;
-            GCK(cudaMalloc(&B.pos, sizeof(double) * 3 * (size_t)np), "particle upload");
-            GCK(cudaMalloc(&B.mass, sizeof(double) * (size_t)np), "particle upload");
-            B.cap = np;
-        }
         GCK(cudaMemcpyAsync(B.pos, pos, sizeof(double) * 3 * (size_t)np, cudaMemcpyHostToDevice, st), "upload");
         GCK(cudaMemcpyAsync(B.mass, mass, sizeof(double) * (size_t)np, cudaMemcpyHostToDevice, st), "upload");
         k_cic<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(np, B.pos, B.mass, lo[0], lo[1], lo[2], 1.0 / B.h, n,
@@ -680,12 +680,13 @@ int grid_build(GridDev &g, int64_t np, const double *pos, const double *mass, do
                bool fp64, cudaStream_t st, std::string &err)
 {
     Builder B;
-    int rc = builder_init(B, g.n, g.h, soft, st, err);
+    int rc = builder_init(B, g.n, g.h, soft, np, st, err);
     if (rc != RT3D_OK) return rc;
     if (fp64)
         GCK(cudaMalloc(&g.tab, sizeof(double) * kGridRec * (size_t)B.n3()), "grid node table");
     else
         GCK(cudaMalloc(&g.tab32, sizeof(float) * kGridRec * (size_t)B.n3()), "grid node table");
+    builder_keep_spectra(B);
     rc = builder_run(B, np, pos, mass, g.lo, mean_subtract, g.tab, g.tab32, st);
     if (rc != RT3D_OK) return rc;
     GCK(cudaStreamSynchronize(st), "grid build");
@@ -749,13 +750,16 @@ int grid_build_box(GridDev &g, int64_t np, const double *pos, const double *mass
             }
     }
     Builder B;
-    int rc = builder_init(B, g.n, g.h, soft, st, err);
+    size_t most = 0;
+    for (const auto &m : cm) most = std::max(most, m.size());
+    int rc = builder_init(B, g.n, g.h, soft, (int64_t)most, st, err);
     if (rc != RT3D_OK) return rc;
     const size_t stride = kGridRec * (size_t)B.n3();
     if (fp64)
         GCK(cudaMalloc(&g.tab, sizeof(double) * stride * (size_t)R * C), "grid node tables");
     else
         GCK(cudaMalloc(&g.tab32, sizeof(float) * stride * (size_t)R * C), "grid node tables");
+    builder_keep_spectra(B);
     for (int j = 0; j < R; ++j)
         for (int q = 0; q < C; ++q) {
             const size_t cell = (size_t)j * C + q;
