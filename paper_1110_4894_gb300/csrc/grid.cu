@@ -575,14 +575,19 @@ static int builder_init(Builder &B, int n, double h, double soft, int64_t np_mos
         GCK(cudaMalloc(&B.pos, sizeof(double) * 3 * (size_t)np_most), "particle upload");
         GCK(cudaMalloc(&B.mass, sizeof(double) * (size_t)np_most), "particle upload");
     }
-    int plane[2] = {P, P}, half[2] = {P, n + 1}, line[1] = {P};
-    const int pd = P * P, pc = P * (n + 1);
-    FCK(cufftPlanMany(&B.r2c, 2, plane, plane, 1, pd, half, 1, pc, CUFFT_D2Z, n), "cufftPlanMany D2Z");
+    // (64-bit sizes: from 813 nodes on the transforms cover more than 2^31 elements)
+    long long plane[2] = {P, P}, half[2] = {P, n + 1}, line[1] = {P};
+    const long long pd = (long long)P * P, pc = (long long)P * (n + 1);
+    size_t work = 0;
+    FCK(cufftCreate(&B.r2c), "cufftCreate");
     B.have_r2c = true;
-    FCK(cufftPlanMany(&B.c2r, 2, plane, half, 1, pc, plane, 1, pd, CUFFT_Z2D, n), "cufftPlanMany Z2D");
+    FCK(cufftMakePlanMany64(B.r2c, 2, plane, plane, 1, pd, half, 1, pc, CUFFT_D2Z, n, &work), "cuFFT plan D2Z");
+    FCK(cufftCreate(&B.c2r), "cufftCreate");
     B.have_c2r = true;
-    FCK(cufftPlanMany(&B.c2c, 1, line, line, pc, 1, line, pc, 1, CUFFT_Z2Z, pc), "cufftPlanMany Z2Z");
+    FCK(cufftMakePlanMany64(B.c2r, 2, plane, half, 1, pc, plane, 1, pd, CUFFT_Z2D, n, &work), "cuFFT plan Z2D");
+    FCK(cufftCreate(&B.c2c), "cufftCreate");
     B.have_c2c = true;
+    FCK(cufftMakePlanMany64(B.c2c, 1, line, line, pc, 1, line, pc, 1, CUFFT_Z2Z, pc, &work), "cuFFT plan Z2Z");
     FCK(cufftSetStream(B.r2c, st), "cufftSetStream");
     FCK(cufftSetStream(B.c2r, st), "cufftSetStream");
     FCK(cufftSetStream(B.c2c, st), "cufftSetStream");
