@@ -143,7 +143,8 @@ typedef struct {
     int64_t launches;     /* kernels launched by the last trace/batch */
     int64_t force_launches;
     int steps;            /* RK4 steps issued */
-    int rays_per_thread, threads_per_block, splits; /* force launch shape used */
+    int rays_per_thread, threads_per_block, splits; /* force launch shape used (rays_per_thread: a
+                             bundle's rays for variants 3 to 5, also where few bundles put one ray on a lane) */
     int variant;          /* pair-sum kernel used: 0 packed, 1 scalar, 2 FP64, 3 bundle, 4 two bundles
                              per thread, 5 two bundles per thread, expanded separations, 6 grid path */
     int cluster;          /* thread-block cluster size along the splits (1: none); the

@@ -1094,7 +1094,8 @@ static int trace_advance(rt3d_ctx *ctx, int n, cudaStream_t st)
     // fields that each ray evaluates for itself: all the stages in one launch
     // (timed traces: kernel by kernel)
     const bool few = T.fp64 && !fs.is_grid && !fs.df.replicated && fs.n <= kFewParticles;
-    if ((fs.is_grid || few) && !T.timed && T.next < stop) {
+    const bool one_launch = (fs.is_grid || few) && !T.timed;
+    if (one_launch && T.next < stop) {
         if (few)
             CK(launch_few_trace(T.tp, fs.df, T.rs, T.next, stop, s.dlam, s.misc, s.counters, st));
         else
@@ -1132,9 +1133,9 @@ static int trace_advance(rt3d_ctx *ctx, int n, cudaStream_t st)
     ctx->stats.launches = T.launches;
     ctx->stats.force_launches = T.flaunch;
     ctx->stats.steps = (T.next + 3) / 4;
-    ctx->stats.rays_per_thread = T.sh.R;
-    ctx->stats.threads_per_block = T.sh.NT;
-    ctx->stats.splits = T.sh.splits;
+    ctx->stats.rays_per_thread = one_launch ? 1 : T.sh.R;
+    ctx->stats.threads_per_block = one_launch ? kTraceRaysNT : (T.sh.lanes ? lanes_threads(T.sh, n_rays) : T.sh.NT);
+    ctx->stats.splits = one_launch ? 1 : T.sh.splits;
     ctx->stats.cluster = T.sh.cl;
     ctx->stats.variant = T.sh.variant;
     // grid path: one field evaluation per ray and stage counts as one

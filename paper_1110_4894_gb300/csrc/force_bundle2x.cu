@@ -79,12 +79,11 @@ static cudaError_t go_lanes(const ForceArgs &A, int group, int splits, cudaStrea
     return launch_overlapped(kern, grid, NT, st, A, group);
 }
 
-// one ray per lane (one tile per split): one-warp blocks while a tile's rays fit
-// one, else four warps, which share the staging of the tile
+// one ray per lane (one tile per split)
 cudaError_t dispatch_lanes(const ForceArgs &A, const ForceShape &sh, bool umass, cudaStream_t st)
 {
     const int group = 2 * sh.NT;
-    const bool one = A.n / sh.R <= 32 / sh.R;
+    const bool one = lanes_threads(sh, A.n) == 32;
     if (sh.R == 5) {
         if (one) return umass ? go_lanes<32, 4, true>(A, group, sh.splits, st) : go_lanes<32, 4, false>(A, group, sh.splits, st);
         return umass ? go_lanes<128, 4, true>(A, group, sh.splits, st) : go_lanes<128, 4, false>(A, group, sh.splits, st);

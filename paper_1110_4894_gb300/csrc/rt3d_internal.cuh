@@ -394,6 +394,10 @@ struct ForceShape {
                   // CTAs' partials in distributed shared memory, one partial per cluster
     int lanes = 0;  // variant 5: one ray per lane (k_force_bundle1), one tile per split
 };
+// threads of a block of k_force_bundle1: one warp while it holds all the bundles,
+// else four warps, which share the staging of a tile
+inline int lanes_threads(const ForceShape &sh, int64_t n_rays) { return n_rays / sh.R <= 32 / sh.R ? 32 : 128; }
+constexpr int kTraceRaysNT = 32;  // threads of a block of the one-launch traces (trace_rays)
 // split partials a shape leaves for the integrator stage
 inline int partial_splits(const ForceShape &sh) { return sh.splits / sh.cl; }
 

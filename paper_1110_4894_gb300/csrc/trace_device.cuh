@@ -451,9 +451,8 @@ __device__ __forceinline__ bool stage_ray(const TraceParams &tp, const DevField 
 // stages in one launch; x3 comes by shuffle.  The bound is FP64: about 150
 // operations per ray and stage on two lanes per SM, in a chain of some sixty.
 // A bundle whose rays are all across stops: results are taken at the crossing,
-// and the stages after it only served other bundles.  Blocks are one warp, which
-// spreads a few hundred warps evenly over the SMs.
-constexpr int kTraceRaysNT = 32;
+// and the stages after it only served other bundles.  Blocks are one warp
+// (kTraceRaysNT), which spreads a few hundred warps evenly over the SMs.
 
 template <class Eval>
 __device__ __forceinline__ void trace_rays(const TraceParams &tp, const RayState &rs, int g0, int g1,

@@ -48,6 +48,28 @@ def test_one_ray_lanes_give_the_same_bits(n_ring, bundles, n, varied, box):
         assert np.array_equal(res[0][k], res[1][k]), k
 
 
+def test_statistics_name_the_block_that_ran():
+    """one-ray lanes run in blocks of one warp (bundles that fit it) or four, two-bundle threads in blocks of 64, and
+    the traces whose rays evaluate the field themselves in blocks of one warp"""
+    import paper_1110_4894_gb300 as P
+    pos, mass, soft, vol = case(517, False, False)
+    shapes = {}
+    for name, opt, bundles in (("warp", {}, 6), ("block", {}, 7), ("threads", dict(splits=3), 7),
+                               ("few", dict(precision=P.FP64), 7), ("grid", {}, 7)):
+        ctx = P.Context(0, **opt)
+        ctx.set_cosmology(0.3, 0.7, 0.7)
+        if name == "grid":
+            ctx.load_grid(0, pos, mass, soft, [-2.0, -2.0, 998.0], 4.0 / 15, 16)
+        else:
+            ctx.load_particles(0, pos[:3] if name == "few" else pos, mass[:3] if name == "few" else mass, soft, **vol)
+        ctx.trace(0, 0.5, 2e-4 * inputs.rng(7).normal(size=(bundles, 2)), n_ring=4, theta_r=5e-6, n_steps=3)
+        st = ctx.stats()
+        ctx.close()
+        shapes[name] = (st["rays_per_thread"], st["threads_per_block"], st["splits"])
+    assert shapes == {"warp": (5, 32, 3), "block": (5, 128, 3), "threads": (5, 64, 3), "few": (1, 32, 1),
+                      "grid": (1, 32, 1)}
+
+
 @pytest.mark.parametrize("box", [False, True])
 def test_captured_trace_replays(box):
     """the overlapped launches of a trace, captured into a CUDA graph and replayed, give the same bits"""
