@@ -69,3 +69,26 @@ def test_many_splits(bundles, n_ring, splits):
         res.append(ctx.trace(0, 0.5, theta, n_ring=n_ring, theta_r=5e-6, n_steps=6)["mu"])
         ctx.close()
     assert np.max(np.abs(res[1] - res[0])) <= 1e-9 * np.max(np.abs(res[0]))
+
+
+# (96 rows in flight: from 256 splits on, where the partials are not added up
+# beforehand, which is above 4864 / 4 rays or in FP64, and up to 152 blocks of 32 rays)
+@pytest.mark.parametrize("precision,bundles", [("mixed", 256), ("mixed", 900), ("fp64", 1), ("fp64", 40), ("fp64", 900)])
+@pytest.mark.parametrize("splits", [256, 287, 288, 289, 480])
+def test_many_splits_in_the_stage(precision, bundles, splits):
+    import paper_1110_4894_gb300 as P
+    per = 256 if precision == "mixed" else 64
+    n = per * splits - 3
+    g = inputs.rng(inputs.BASE_SEED + 133)
+    pos = inputs.quantize(np.array([0.0, 0.0, 1000.0]) + 0.5 * g.normal(size=(n, 3)))
+    theta = np.array([3e-4, -2e-4]) + 2e-4 * g.normal(size=(bundles, 2))
+    res = []
+    for s in (64, splits):
+        ctx = P.Context(0, precision=P.FP64 if precision == "fp64" else P.MIXED, splits=s)
+        ctx.set_cosmology(0.3, 0.7, 0.7)
+        ctx.load_particles(0, pos, 1e9 * 33280 / n, 0.05)
+        res.append(ctx.trace(0, 0.5, theta, n_ring=4, theta_r=5e-6, n_steps=6)["mu"])
+        used = ctx.stats()["splits"]
+        ctx.close()
+    assert used == splits
+    assert np.max(np.abs(res[1] - res[0])) <= 1e-9 * np.max(np.abs(res[0]))
