@@ -170,7 +170,16 @@ def run_cones(args):
 GRID_FLOPS_PER_RAY = 4 * 2 * (16 * 8 + 16 + 4) + 100
 GRID_ROOFLINE_NOTE = ("k_grid_eval32 gathers its node records mostly from L1/L2 and is bound by that latency, "
                       "neither by HBM nor by the FP32 pipe (low frac); a trace's own bound on the grid path is "
-                      "the FP64 integrator stage")
+                      "the FP64 of the integrator stages")
+
+
+def grid_eval_ms(ctx, trace):
+    """mean time of the stage-by-stage evaluation kernel, k_grid_eval32: ctx has time_kernels=1, which takes a
+    grid trace kernel by kernel (an ordinary one is a single launch, k_grid_trace)"""
+    trace(ctx)
+    trace(ctx)
+    st = ctx.stats()
+    return st["force_ms"] / max(1, st["force_launches"])
 
 
 def run_grid(args):
@@ -195,7 +204,7 @@ def run_grid(args):
     lo = [-half, -half, cfg["chi_l"] - half]
     kw = trace_kw(cfg)
     nb = cfg["theta"].shape[0]
-    ctx = P.Context(0, precision=P.MIXED, time_kernels=1)
+    ctx = P.Context(0, precision=P.MIXED)
     ctx.set_cosmology(*cfg["cosmo"])
     t0 = time.perf_counter()
     ctx.load_grid(0, cfg["pos"], cfg["mass"], cfg["soft"], lo, h, n, n_int=2)
@@ -209,8 +218,11 @@ def run_grid(args):
     stream = torch.cuda.current_stream(dev)
     sp = stream.cuda_stream
 
+    def trace(c):
+        c.trace_device(sp, 0, cfg["z_s"], nb, d_theta.data_ptr(), d_bout.data_ptr(), **kw)
+
     def step():
-        ctx.trace_device(sp, 0, cfg["z_s"], nb, d_theta.data_ptr(), d_bout.data_ptr(), **kw)
+        trace(ctx)
         ctx.histogram_device(sp, nb, d_bout.data_ptr(), d_counts.data_ptr(), d_wfix.data_ptr(), d_scal.data_ptr(),
                              **HIST)
 
@@ -218,7 +230,7 @@ def run_grid(args):
         step()
     torch.cuda.synchronize(dev)
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
-    eval_ms, eval_launches, evals, launches = 0.0, 0, 0.0, 0
+    evals, launches = 0.0, 0
     with ClockSampler(0) as clk:
         for k in range(args.steps):
             flush.zero_()
@@ -226,13 +238,16 @@ def run_grid(args):
             step()
             ev[k][1].record(stream)
             st = ctx.stats()
-            eval_ms += st["force_ms"]
-            eval_launches += st["force_launches"]
             evals += st["interactions"]  # ray-stage field evaluations on the grid path
             launches += st["launches"] + 2
     clocks = clk.summary()
     dev_s = sum(a.elapsed_time(b) for a, b in ev) / 1e3
     mu_grid = d_bout.view(nb, 6)[:, 0].cpu().numpy()
+    ct = P.Context(0, precision=P.MIXED, time_kernels=1)
+    ct.set_cosmology(*cfg["cosmo"])
+    ct.load_grid(0, cfg["pos"], cfg["mass"], cfg["soft"], lo, h, n, n_int=2)
+    eval_ms = grid_eval_ms(ct, trace)
+    ct.close()
     # the direct sum on the same bundles, for the grid's smoothing error
     cd = P.Context(0, precision=P.MIXED, autotune=1)
     cd.set_cosmology(*cfg["cosmo"])
@@ -245,7 +260,7 @@ def run_grid(args):
     c64.load_grid(0, cfg["pos"], cfg["mass"], cfg["soft"], lo, h, n, n_int=2)
     mu64 = c64.trace(0, cfg["z_s"], cfg["theta"], **kw)["mu"]
     dmu64 = float(np.max(np.abs(mu_grid / mu64 - 1)))
-    per_launch_s = eval_ms / 1e3 / max(1, eval_launches)
+    per_launch_s = eval_ms / 1e3
     flops_per_launch = nb * (1 + cfg["n_ring"]) * GRID_FLOPS_PER_RAY
     out = {"metric": "ray bundles/s (grid path)", "value": nb * args.steps / dev_s, "unit": "bundles/s",
            "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1e3 * dev_s / args.steps,
@@ -257,6 +272,7 @@ def run_grid(args):
            "roofline": {"bound": "alu", "achieved": flops_per_launch / per_launch_s / 1e12, "peak": FP32_PEAK / 1e12,
                         "unit": "TFLOP/s", "frac": flops_per_launch / per_launch_s / FP32_PEAK, "traffic": None,
                         "kernel": "k_grid_eval32", "avg_launch_ms": per_launch_s * 1e3,
+                        "of": "a trace kernel by kernel; the timed steps are one launch each (k_grid_trace)",
                         "note": GRID_ROOFLINE_NOTE},
            "grid_vs_direct_sum": {"median_abs_dmu_over_mu": float(np.median(dmu)),
                                   "max_abs_dmu_over_mu": float(np.max(dmu))},
@@ -282,7 +298,7 @@ def run_prism(args):
     cfg = inputs.config_prism(n_steps=args.rk4_steps or 1000)
     n, cubes = cfg["grid_n"], cfg["cubes"]
     nb = cfg["theta"].shape[0]
-    ctx = P.Context(0, precision=P.MIXED, time_kernels=1)
+    ctx = P.Context(0, precision=P.MIXED)
     ctx.set_cosmology(*cfg["cosmo"])
     t0 = time.perf_counter()
     ctx.load_grid_box(0, cfg["pos"], cfg["mass"], cfg["soft"], cfg["L"], cfg["rot"], cfg["shift"], cubes, n,
@@ -297,8 +313,11 @@ def run_prism(args):
     stream = torch.cuda.current_stream(dev)
     sp = stream.cuda_stream
 
+    def trace(c):
+        c.trace_device(sp, 0, cfg["z_s"], nb, d_theta.data_ptr(), d_bout.data_ptr(), **kw)
+
     def step():
-        ctx.trace_device(sp, 0, cfg["z_s"], nb, d_theta.data_ptr(), d_bout.data_ptr(), **kw)
+        trace(ctx)
         ctx.histogram_device(sp, nb, d_bout.data_ptr(), d_counts.data_ptr(), d_wfix.data_ptr(), d_scal.data_ptr(),
                              **HIST)
 
@@ -306,21 +325,25 @@ def run_prism(args):
         step()
     torch.cuda.synchronize(dev)
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
-    eval_ms, eval_launches, evals, launches = 0.0, 0, 0.0, 0
+    evals, launches = 0.0, 0
     with ClockSampler(0) as clk:
         for k in range(args.steps):
             ev[k][0].record(stream)
             step()
             ev[k][1].record(stream)
             st = ctx.stats()
-            eval_ms += st["force_ms"]
-            eval_launches += st["force_launches"]
             evals += st["interactions"]
             launches += st["launches"] + 2
     clocks = clk.summary()
     dev_s = sum(a.elapsed_time(b) for a, b in ev) / 1e3
     scal = d_scal.cpu().numpy()
     res = d_bout.view(nb, 6).cpu().numpy()
+    ct = P.Context(0, precision=P.MIXED, time_kernels=1)
+    ct.set_cosmology(*cfg["cosmo"])
+    ct.load_grid_box(0, cfg["pos"], cfg["mass"], cfg["soft"], cfg["L"], cfg["rot"], cfg["shift"], cubes, n,
+                     n_int=2, mean_subtract=True)
+    eval_ms = grid_eval_ms(ct, trace)
+    ct.close()
     # the FP64 grid path on the first bundles: the mixed path's FP32 interpolation error
     k = min(nb, args.fp64_bundles)
     c64 = P.Context(0, precision=P.FP64)
@@ -329,7 +352,7 @@ def run_prism(args):
                       n_int=2, mean_subtract=True)
     mu64 = c64.trace(0, cfg["z_s"], cfg["theta"][:k], **kw)["mu"]
     dmu64 = float(np.max(np.abs(res[:k, 0] / mu64 - 1)))
-    per_launch_s = eval_ms / 1e3 / max(1, eval_launches)
+    per_launch_s = eval_ms / 1e3
     flops_per_launch = nb * (1 + cfg["n_ring"]) * GRID_FLOPS_PER_RAY
     out = {"metric": "ray bundles/s (grid path, replicated box)", "value": nb * args.steps / dev_s,
            "unit": "bundles/s", "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
@@ -345,6 +368,7 @@ def run_prism(args):
            "roofline": {"bound": "alu", "achieved": flops_per_launch / per_launch_s / 1e12, "peak": FP32_PEAK / 1e12,
                         "unit": "TFLOP/s", "frac": flops_per_launch / per_launch_s / FP32_PEAK, "traffic": None,
                         "kernel": "k_grid_eval32", "avg_launch_ms": per_launch_s * 1e3,
+                        "of": "a trace kernel by kernel; the timed steps are one launch each (k_grid_trace)",
                         "note": GRID_ROOFLINE_NOTE},
            "mixed_vs_fp64_grid": {"bundles": k, "max_abs_dmu_over_mu": dmu64},
            "mupdf": {"bundles_binned": int(scal[0]), "mean_w": float(scal[6]), "sigma_w": float(scal[7]),
