@@ -1093,7 +1093,7 @@ static int trace_advance(rt3d_ctx *ctx, int n, cudaStream_t st)
     const int stop = std::min(T.total, T.next + n);
     // fields that each ray evaluates for itself: all the stages in one launch
     // (timed traces: kernel by kernel)
-    const bool few = T.fp64 && !fs.is_grid && !fs.df.replicated && fs.n <= kFewParticles;
+    const bool few = T.fp64 && !fs.is_grid && !fs.df.replicated && few_in_one_launch(fs.n, n_rays);
     const bool one_launch = (fs.is_grid || few) && !T.timed;
     if (one_launch && T.next < stop) {
         if (few)

@@ -455,7 +455,8 @@ inline double partial_mass_factor(const DevField &f, const ForceShape &sh)
     return sh.umass ? f.m_uniform : 1.0;
 }
 // RK4 stages [g0, g1) of an FP64 trace through an isolated field of few particles
-constexpr int kFewParticles = 64;
+constexpr int kFewParticles = 64, kFewAlways = 22;
+bool few_in_one_launch(int64_t n_particles, int64_t n_rays);
 cudaError_t launch_few_trace(const TraceParams &tp, const DevField &f, const RayState &rs, int g0, int g1,
                              const double *d_dlam, const double *d_misc, unsigned long long *d_counters,
                              cudaStream_t st);

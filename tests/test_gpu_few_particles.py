@@ -61,3 +61,27 @@ def test_few_particles_in_pieces(cosmo):
     torch.cuda.synchronize()
     ctx.close()
     assert torch.equal(out[0], out[1])
+
+
+# one launch up to 22 particles, and up to 64 from 16 rays an SM on (2432 on GB300's 152)
+@pytest.mark.parametrize("n,bundles,one", [(22, 3, True), (23, 3, False), (23, 486, False), (23, 487, True),
+                                           (64, 486, False), (64, 487, True), (65, 487, False)])
+def test_where_one_launch_takes_over(n, bundles, one):
+    import torch
+
+    import paper_1110_4894_gb300 as P
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    bundles = bundles * sms // 152 + (bundles == 487 and sms != 152)
+    g = inputs.rng(inputs.BASE_SEED + n)
+    pos = inputs.quantize(np.array([0.0, 0.0, 1000.0]) + 0.3 * g.normal(size=(n, 3)))
+    theta = 3e-4 * g.normal(size=(bundles, 2))
+    kw = dict(n_ring=4, theta_r=5e-6, schedule=1, n_steps=60, lens_chi=1000.0, asinh_s=0.05)
+    res = []
+    for timed in (0, 1):
+        ctx = P.Context(0, precision=P.FP64, time_kernels=timed)
+        ctx.set_cosmology(0.3, 0.7, 0.7)
+        ctx.load_particles(0, pos, 1e13 / n, 0.03)
+        res.append(ctx.trace(0, 0.5, theta, **kw))
+        assert (ctx.stats()["threads_per_block"] == 32) == (one and not timed)
+        ctx.close()
+    assert np.max(np.abs(res[0]["mu"] / res[1]["mu"] - 1)) < 1e-10
