@@ -44,3 +44,43 @@ def test_grid_build_without_room_for_the_spectra():
         ctx.close()
     assert np.max(np.abs(res[0])) > 0.0
     assert np.all(np.abs(res[1] - res[0]) <= 1e-11 * np.max(np.abs(res[0]), axis=0))
+
+
+@pytest.mark.parametrize("bad", [None, "pos", "mass", "soft", "box"])
+def test_load_beside_a_field_that_leaves_no_room(bad):
+    """a new field whose upload does not fit beside the old one: valid particles take its place, invalid ones are
+    found on the host before it goes.  The old one holds 16 bytes or more a particle, an upload takes 32 to 40"""
+    import paper_1110_4894_gb300 as P
+    n = 1 << 22
+    g = inputs.rng(inputs.BASE_SEED + 82)
+    L = inputs.box_length(8.0)
+    pos, mass, soft = g.random((n, 3)) * L * 0.999, g.uniform(1e8, 2e8, n), g.uniform(0.01, 0.02, n)
+    old = np.tile(pos, (4, 1))
+    vol = dict(replicated=True, box_length=L, rot=np.eye(3, dtype=np.int32)[None], shift=np.zeros((1, 3)))
+    at = g.random((50, 3))
+    ctx = P.Context(0)
+    ctx.load_particles(0, pos, mass, soft, **vol)
+    want = ctx.potential(0, at)
+    ctx.load_particles(0, old, 1e8, 0.02)
+    before = ctx.potential(0, at)
+    if bad == "pos":
+        pos[n // 2, 1] = np.inf
+    elif bad == "mass":
+        mass[n - 1] = -1.0
+    elif bad == "soft":
+        soft[n // 3] = np.nan
+    elif bad == "box":
+        pos[n - 1, 2] = 1.5 * L
+    filler = leave(20 * n)
+    if bad is None:
+        ctx.load_particles(0, pos, mass, soft, **vol)
+        assert np.array_equal(ctx.potential(0, at), want)
+    else:
+        message = {"pos": "non-finite", "mass": "masses must", "soft": "softening", "box": "outside [0, L]"}[bad]
+        with pytest.raises(P.Rt3dError) as e:
+            ctx.load_particles(0, pos, mass, soft, **vol)
+        assert message in str(e.value)
+        assert np.array_equal(ctx.potential(0, at), before)
+    del filler
+    release()
+    ctx.close()
