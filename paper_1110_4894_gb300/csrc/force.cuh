@@ -1137,7 +1137,6 @@ __global__ void __launch_bounds__(NT, 1) k_force_bundle1(ForceArgs A, int group)
     __shared__ int s_rmin, s_rmax;
     const DevField &f = A.f;
     const int tid = threadIdx.x, split = blockIdx.y;
-    let_next_start();
     // the tile's particles are the field's: they are read ahead of the wait
     const int64_t p0 = (int64_t)split * kTile;
     const int cnt = (int)min((int64_t)kTile, f.n - p0);
@@ -1279,7 +1278,6 @@ __global__ void __launch_bounds__(NT) k_force_bundle(ForceArgs A)
 template <int R, int NT, bool REPL, bool PEPS>
 __global__ void __launch_bounds__(NT) k_force_fp64(ForceArgs A)
 {
-    let_next_start();
     wait_for_previous();
     if (A.gate && *A.gate == 0ull) return;
     __shared__ double4_16a s_p[kTile64];
