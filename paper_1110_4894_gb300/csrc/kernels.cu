@@ -358,15 +358,16 @@ cudaError_t launch_stage(const TraceParams &tp, const DevField &f, RayState rs, 
 //
 // One launch costs each ray its particles in turn (4.4 + 0.65 us a particle and
 // stage while the warps have a scheduler each), the two kernels of a stage 18 us
-// and more from some 10,000 rays on.  ms for 50 steps in one launch / by stages:
-// 66 bundles of 5: 8 particles 1.9 / 3.8, 22 3.75 / 3.98, 28 4.5 / 4.1, 40 6.1 /
-// 3.9, 64 9.2 / 4.2; 512 bundles: 28 4.5 / 4.1, 40 6.1 / 8.9; 2048: 22 3.8 / 11.4,
-// 40 6.1 / 9.2, 64 9.17 / 9.22; 32,768: 22 32 / 40, 64 81 / 86.  So the stages run
-// by themselves from 23 particles on where there are fewer than 16 rays an SM.
+// and more from a few thousand rays on.  ms for 50 steps in one launch / by
+// stages: 66 bundles of 5: 8 particles 1.9 / 3.6, 22 3.6 / 3.9, 32 4.9 / 3.9, 64
+// 8.8 / 3.8; 1024 bundles: 22 3.6 / 3.8, 32 4.9 / 5.0, 64 8.8 / 6.3; 2048: 22 3.6 /
+// 5.0, 32 4.9 / 6.3, 64 8.8 / 9.0; 4096: 64 11.9 / 14.4; 32,768: 22 33 / 39, 64 81 /
+// 85.  So the stages run by themselves from 23 particles on where there are fewer
+// than 64 rays an SM.
 bool few_in_one_launch(int64_t n_particles, int64_t n_rays)
 {
     return n_particles <= kFewAlways ||
-           (n_particles <= kFewParticles && n_rays >= 16 * (int64_t)device_sm_count());
+           (n_particles <= kFewParticles && n_rays >= 64 * (int64_t)device_sm_count());
 }
 
 template <bool PEPS>

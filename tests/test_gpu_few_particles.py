@@ -63,15 +63,15 @@ def test_few_particles_in_pieces(cosmo):
     assert torch.equal(out[0], out[1])
 
 
-# one launch up to 22 particles, and up to 64 from 16 rays an SM on (2432 on GB300's 152)
-@pytest.mark.parametrize("n,bundles,one", [(22, 3, True), (23, 3, False), (23, 486, False), (23, 487, True),
-                                           (64, 486, False), (64, 487, True), (65, 487, False)])
+# one launch up to 22 particles, and up to 64 from 64 rays an SM on (9728 on GB300's 152)
+@pytest.mark.parametrize("n,bundles,one", [(22, 3, True), (23, 3, False), (23, 1945, False), (23, 1946, True),
+                                           (64, 1945, False), (64, 1946, True), (65, 1946, False)])
 def test_where_one_launch_takes_over(n, bundles, one):
     import torch
 
     import paper_1110_4894_gb300 as P
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    bundles = bundles * sms // 152 + (bundles == 487 and sms != 152)
+    bundles = bundles * sms // 152 + (bundles == 1946 and sms != 152)
     g = inputs.rng(inputs.BASE_SEED + n)
     pos = inputs.quantize(np.array([0.0, 0.0, 1000.0]) + 0.3 * g.normal(size=(n, 3)))
     theta = 3e-4 * g.normal(size=(bundles, 2))
@@ -84,4 +84,6 @@ def test_where_one_launch_takes_over(n, bundles, one):
         res.append(ctx.trace(0, 0.5, theta, **kw))
         assert (ctx.stats()["threads_per_block"] == 32) == (one and not timed)
         ctx.close()
-    assert np.max(np.abs(res[0]["mu"] / res[1]["mu"] - 1)) < 1e-10
+    # (of 1 / mu, the Jacobian's determinant, as some of these many bundles may lie near a critical line)
+    a, b = 1 / res[0]["mu"], 1 / res[1]["mu"]
+    assert np.all(np.abs(a - b) <= 1e-10 * (1 + np.abs(b)))
