@@ -1128,7 +1128,7 @@ __global__ void __launch_bounds__(NT, TPSM / NT) k_force_bundle2x(ForceArgs A)
 // two-bundle kernel, so the results are the same bits.  One tile per block
 // (blockIdx.y); a block holds NT / NR whole bundles.
 template <int NT, int NRING, bool REPL, bool PEPS, bool UMASS>
-__global__ void __launch_bounds__(NT, 1) k_force_bundle1(ForceArgs A, int group)
+__global__ void __launch_bounds__(NT, 1) k_force_bundle1(ForceArgs A, int group, bool early)
 {
     constexpr int NR = NRING + 1, BPB = NT / NR;
     __shared__ float4 s_p[kTile];
@@ -1137,6 +1137,7 @@ __global__ void __launch_bounds__(NT, 1) k_force_bundle1(ForceArgs A, int group)
     __shared__ int s_rmin, s_rmax;
     const DevField &f = A.f;
     const int tid = threadIdx.x, split = blockIdx.y;
+    if (early) let_next_start();
     // the tile's particles are the field's: they are read ahead of the wait
     const int64_t p0 = (int64_t)split * kTile;
     const int cnt = (int)min((int64_t)kTile, f.n - p0);

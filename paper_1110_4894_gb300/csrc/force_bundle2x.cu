@@ -76,7 +76,9 @@ static cudaError_t go_lanes(const ForceArgs &A, int group, int splits, cudaStrea
     const dim3 grid((unsigned)(full * ((group + BPB - 1) / BPB) + (rest + BPB - 1) / BPB), (unsigned)splits);
     const auto kern = repl ? (peps ? k_force_bundle1<NT, NRING, true, true, UMASS> : k_force_bundle1<NT, NRING, true, false, UMASS>)
                            : (peps ? k_force_bundle1<NT, NRING, false, true, UMASS> : k_force_bundle1<NT, NRING, false, false, UMASS>);
-    return launch_overlapped(kern, grid, NT, st, A, group);
+    // (rt3d_internal.cuh says why)
+    const bool early = !repl && (int64_t)grid.x * grid.y <= device_sm_count();
+    return launch_overlapped(kern, grid, NT, st, A, group, early);
 }
 
 // one ray per lane (one tile per split)

@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(32) k_prism(TraceParams tp, DevField f, RaySta
                                               const unsigned long long *cnt, double *prism)
 {
     __shared__ double s_q[kPrismBundles][10 * kCorners];
+    let_next_start();
     wait_for_previous();
     if (step >= tp.n_steps && cnt[(step - 1) & 1] == 0ull) return;  // every ray is across
     const int k = threadIdx.x / kCorners;
@@ -161,6 +162,7 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge(float2 *partials, int S
 {
     __shared__ float2 s_v[kMergeTiles][kMergeRows][kMergeRays];  // (x, y) of a row; y becomes w
     __shared__ float s_t[2][kMergeRows + 1][kMergeRays];         // high sums before each row, and after the last
+    let_next_start();
     wait_for_previous();
     if (step >= n_steps && cnt[(step - 1) & 1] == 0ull) return;  // every ray is across
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, o = blockIdx.y;
@@ -255,7 +257,8 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(TraceParams tp, DevFiel
         const int64_t pitch = 4 * rs.n_rays;
         float2 buf[G][kRows];
         // (rows past the last split are zeros, which leave the sum as it is; read
-        // from L2, where k_merge's row 0 is whatever its blocks left in this SM's L1)
+        // from L2: this block may have started while k_merge, on the same SM, had
+        // the lines of row 0 in L1)
         const auto load = [&](int g, int s0) {
 #pragma unroll
             for (int r = 0; r < kRows; ++r, src += pitch)

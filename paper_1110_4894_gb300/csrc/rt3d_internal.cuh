@@ -196,22 +196,27 @@ __device__ __forceinline__ void prism_field_hess(const T lo[3], const T hi[3], c
 // ---------------------------------------------------------------------------
 // The short kernels of a trace follow one another some thousand times, and the
 // gap between two of them (2.7 us, against 4 to 8 us of work in a small trace)
-// is launch latency (4 bundles through 5000 particles, 200 steps: 18.1 -> 13.4
+// is launch latency (4 bundles through 5000 particles, 200 steps: 18.1 -> 12.6
 // ms).  Launched this way, a kernel's blocks may start as soon as every block of
-// the kernel before it in the stream has ended; it must call wait_for_previous
-// before it reads what an earlier kernel of the stream wrote, or writes anything.
-// The wait returns when the kernel before is complete and its writes are visible;
-// as that one waited too, so is every earlier kernel.  In a kernel launched the
-// ordinary way the call does nothing.
-// (No kernel lets the next one start before its own blocks have ended, by
-// griddepcontrol.launch_dependents: the blocks that then wait beside the running
-// ones are packed several to an SM, and the FP64 kernels of a mid-size trace run
-// on part of the SMs.  30 steps with that / launched the ordinary way / as here:
-// 66 bundles through 20,000 particles 3.85 / 3.85 / 2.80 ms, 512 through 2000 4.4 /
-// 3.7 / 2.7, 2048 through 300 5.1 / 3.6 / 2.6; mean-subtracted boxes, where a third
-// kernel waits: 256 through 5000 11.2 / 7.2 / 5.8, 1024 of 8 rays through 500 20.5 /
-// 7.4 / 6.0; FP64, 66 through 300 3.56 / 3.85 / 2.73.  Larger traces: the same.)
+// the kernel before it in the stream has ended, or has called let_next_start; it
+// must call wait_for_previous before it reads what an earlier kernel of the stream
+// wrote, or writes anything.  The wait returns when the kernel before is complete
+// and its writes are visible; as that one waited too, so is every earlier kernel.
+// In a kernel launched the ordinary way both calls do nothing.
+//
+// Blocks that wait beside the running ones are packed several to an SM, and the
+// FP64 stage of a mid-size trace then runs on part of the SMs.  So the stage
+// kernels and k_force_fp64 never let the next one in, k_force_bundle1 does where
+// its blocks leave every SM room (and no prism kernel comes in between), and the
+// short k_prism and k_merge do.  30 steps with all of them letting the next one in
+// / launched the ordinary way / as here: 66 bundles through 20,000 particles 3.85 /
+// 3.85 / 2.85 ms, 512 through 2000 4.4 / 3.7 / 2.75, 2048 through 300 5.1 / 3.6 / 2.6;
+// mean-subtracted boxes: 256 through 5000 13.2 / 7.2 / 5.8, 1024 of 8 rays through
+// 500 20.5 / 7.4 / 6.0; FP64, 66 through 300 3.56 / 3.85 / 2.73.  Larger traces: the
+// same.  4 bundles through 5000 particles, 200 steps, with / here / none letting the
+// next one in: 13.3 / 12.6 / 13.0.
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... P, typename... A>
 inline cudaError_t launch_overlapped(void (*kern)(P...), dim3 grid, int threads, cudaStream_t st, const A &...args)
