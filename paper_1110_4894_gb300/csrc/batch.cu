@@ -9,7 +9,7 @@
 // phase opens the cone's next one.  Cones wait for nobody but themselves, so the
 // end of one cone's stage is filled with others' items, and FP64 stage items run
 // beside FP32 pair sums.  (With a barrier of the whole grid after each phase, 48
-// cones of 1e3-2e5 particles took 173 ms, 157 now.)  A cone whose rays are all across, or whose steps are used up, is done.
+// cones of 1e3-2e5 particles took 173 ms, 157 without; 149 with ragged blocks paired.)  A cone whose rays are all across, or whose steps are used up, is done.
 // A block without work waits for an event (a phase opened, a cone done) at most
 // as long as the %globaltimer watchdog allows: on expiry the kernel sets an error
 // word and returns, and the host reports RT3D_ETIMEOUT.  A block that holds an

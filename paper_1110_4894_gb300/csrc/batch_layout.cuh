@@ -35,7 +35,6 @@ struct BatchArgs {
     int n_cones;
     const int4 *items;     // (cone, ray block, split, kind); split -1: the prism records of a
                            // block of NT bundles; kind 1: grid evaluation of a ray block
-    int64_t n_items;
     const int *order;      // the cones, most expensive first
     const int *rb2cone;    // cone of each padded ray block
     int64_t T;             // padded ray count
@@ -47,15 +46,14 @@ struct BatchArgs {
     double *bout;
 };
 
-inline BatchArgs make_batch_args(void *cones, int n_cones, const int4 *items, int64_t n_items, const int *order,
-                                 const int *rb2cone, int64_t T, int RB, int g_end, unsigned *bar, int *err, double watchdog_s,
+inline BatchArgs make_batch_args(void *cones, int n_cones, const int4 *items, const int *order, const int *rb2cone, int64_t T,
+                                 int RB, int g_end, unsigned *bar, int *err, double watchdog_s,
                                  double *bout)
 {
     BatchArgs A;
     A.cones = (BatchCone *)cones;
     A.n_cones = n_cones;
     A.items = items;
-    A.n_items = n_items;
     A.order = order;
     A.rb2cone = rb2cone;
     A.T = T;

@@ -318,7 +318,8 @@ constexpr int kMp2NT = 64;
 // Only the particles on the plane are staged (in their order), so that a plane
 // costs its own particles and not the whole replica's; what is left per plane is
 // the look at every particle.  524,288 particles, 4096 bundles to z = 0.5: 115.1
-// -> 69.1 ms for two planes per replica; one per replica takes 59.2.
+// -> 69.1 ms for two planes per replica (68.4 with the 32-bit replica map); one per
+// replica takes 59.2.
 // (rings of 4 bounded for 8 blocks per SM, 128 registers, as fast as 7 and 5 %
 // faster than 6; rings of 8, whose accumulators need more, for 4)
 template <int NRING, bool REPL, bool PEPS, bool UMASS>
