@@ -37,7 +37,7 @@ inline int64_t rays_per_block(const ForceShape &sh)
 // What rt3d_load_particles asks of its inputs, and what it needs to know of
 // them, in one pass over the device copies.  (It replaced host loops over the
 // particles and a reduction in a single block: 2^20 particles loaded, traced
-// and binned took 79.9 ms with those, 73.9 without; 2^24 particles load in 8 ms, 134
+// and binned took 79.9 ms with those, 73.9 without; 2^24 particles load in 10 ms, 134
 // before.)
 struct FieldScan {
     double lo[3], hi[3], mmax, msum;
@@ -499,6 +499,18 @@ static const char *check_volume(const rt3d_volume *vol)
     return nullptr;
 }
 
+// A byte of every page of a host array, ahead of its copy to the device.  On a
+// GB300 machine (Grace, 64 KB pages) pageable arrays that the host had not read
+// since the last load, seconds before, were copied at 2 GB/s: 2^24 particles took
+// 190-390 ms to load between two traces.  With the pages touched (1.5 ms) the copy
+// takes 3 ms and the load 10; the loops over the particles that checked them on the
+// host, 134 ms, had done that in passing.
+static void touch_pages(const void *p, size_t bytes)
+{
+    const volatile char *c = static_cast<const volatile char *>(p);
+    for (size_t i = 0; i < bytes; i += 4096) (void)c[i];
+}
+
 extern "C" int rt3d_load_particles(rt3d_ctx *ctx, int field_id, int64_t n, const double *pos, const double *mass,
                                    const double *soft, int soft_pp, const rt3d_volume *vol)
 {
@@ -557,6 +569,9 @@ extern "C" int rt3d_load_particles(rt3d_ctx *ctx, int field_id, int64_t n, const
             double(*part)[7] = reinterpret_cast<double(*)[7]>(d_part);
             double *chain = d_part + 7 * kScanBlocks;
             const int blocks = (int)std::min<int64_t>((n + kScanThreads - 1) / kScanThreads, kScanBlocks);
+            touch_pages(pos, 3 * n * sizeof(double));
+            touch_pages(mass, n * sizeof(double));
+            if (soft_pp) touch_pages(soft, n * sizeof(double));
             if (cudaMemcpyAsync(d_pos, pos, 3 * n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
                 cudaMemcpyAsync(d_mass, mass, n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
                 cudaMemcpyAsync(d_soft, soft, (soft_pp ? n : 1) * sizeof(double), cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
